@@ -70,8 +70,8 @@ def headline_config(N, T, substeps, dt, A, world):
 
 # The translation unit of the forward kernels (the dominant kernel of the
 # headline): its .cu file and the headers of csrc/ it includes.
-FORWARD_TU = ("brax_device.cuh", "brax_forward.cu", "brax_kernels.h", "brax_pair.cuh", "brax_params.h",
-              "brax_physics.cuh")
+FORWARD_TU = ("brax_device.cuh", "brax_kernels.h", "brax_limb.cu", "brax_limb.cuh", "brax_pair.cuh",
+              "brax_params.h", "brax_physics.cuh")
 
 
 def kernel_sources_digest():

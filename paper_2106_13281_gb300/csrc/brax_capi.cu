@@ -64,6 +64,48 @@ struct Rejected {
   } while (0)
 
 // Validate a descriptor and flatten it into the parameter blob.
+// Whether the system has the limb layout's shape (brax_limb.cuh), and which
+// body is which: one root whose L children (L a power of two) each have one
+// child of their own and nothing else, every body of at most two plane points
+// on z-up ground, and all upper (and all lower) bodies alike but for their
+// geometry (offsets, frames, point positions).
+void find_limbs(SysP& S, const std::vector<BodyP>& bodies, const std::vector<PlaneP>& planes) {
+  S.n_limbs = 0;
+  int root = -1;
+  for (int b = 0; b < S.B; ++b)
+    if (!(bodies[b].flags & kHasParent)) {
+      if (root >= 0) return;
+      root = b;
+    }
+  if (root < 0 || !S.flat) return;
+  const BodyP& r = bodies[root];
+  const int L = r.n_children;
+  if (L < 1 || L > BRAX_MAX_CHILDREN || (L & (L - 1)) || S.B != 1 + 2 * L) return;
+  for (int l = 0; l < L; ++l) {
+    const int u = r.children[l];
+    if (bodies[u].n_children != 1) return;
+    S.limb_upper[l] = u;
+    S.limb_lower[l] = bodies[u].children[0];
+  }
+  auto alike = [&](const BodyP& a, const BodyP& b) {
+    bool ok = a.inv_mass == b.inv_mass && a.flags == b.flags && a.k == b.k && a.c == b.c && a.ka == b.ka &&
+              a.ca == b.ca && a.kl == b.kl && a.lo[0] == b.lo[0] && a.hi[0] == b.hi[0] && a.gear[0] == b.gear[0] &&
+              (a.act[0] >= 0) == (b.act[0] >= 0) && a.n_children == b.n_children && a.n_points == b.n_points &&
+              a.n_points <= 2;
+    for (int i = 0; i < 3; ++i) ok = ok && a.inv_I[i] == b.inv_I[i];
+    for (int i = 0; ok && i < a.n_points; ++i)
+      ok = a.pt[i].r == b.pt[i].r && a.pt[i].mu == b.pt[i].mu && a.pt[i].e == b.pt[i].e &&
+           planes[a.pt[i].plane].p0[2] == planes[b.pt[i].plane].p0[2];
+    return ok;
+  };
+  for (int l = 0; l < L; ++l)
+    if (bodies[S.limb_lower[l]].n_children != 0 || !alike(bodies[S.limb_upper[l]], bodies[S.limb_upper[0]]) ||
+        !alike(bodies[S.limb_lower[l]], bodies[S.limb_lower[0]]))
+      return;
+  S.limb_root = root;
+  S.n_limbs = L;
+}
+
 std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int* P_out) {
   REQUIRE(d.version == 1 || d.version == BRAX_DESC_VERSION, "version: expected 1 or BRAX_DESC_VERSION");
   // a version-1 descriptor ends before the variant fields: they are off
@@ -444,6 +486,7 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
   S.iso = 1;
   for (int b = 0; b < S.B; ++b)
     S.iso = S.iso && bodies[b].inv_I[0] == bodies[b].inv_I[1] && bodies[b].inv_I[1] == bodies[b].inv_I[2];
+  find_limbs(S, bodies, planes);
   const double h = (double)d.dt / d.substeps;
   S.h = (float)h;
   S.beta_h = (float)(d.baumgarte / h);
@@ -509,6 +552,7 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
       std::memcpy(blob.data() + base_bytes + sizeof(SysP2) + b * sizeof(BodyP2), &q, sizeof(q));
     }
   }
+  if (!paired) S.n_limbs = 0;
   std::memcpy(blob.data(), &S, sizeof(SysP));
   std::memcpy(blob.data() + blob_bodies_off(), bodies.data(), sizeof(BodyP) * B);
   if (Pb) std::memcpy(blob.data() + blob_pairs_off(B), pairs.data(), sizeof(PairP) * Pb);
@@ -562,6 +606,7 @@ int pool_acquire(int device, const std::vector<unsigned char>& blob) {
   if (off + bytes > kPoolBytes) return -1;
   cudaError_t e = upload_pool_forward(off, blob.data(), blob.size());
   if (e == cudaSuccess) e = upload_pool_backward(off, blob.data(), blob.size());
+  if (e == cudaSuccess) e = upload_pool_limb(off, blob.data(), blob.size());
   if (e != cudaSuccess) return -2 - (int)e;
   g_pool.push_back(PoolRange{device, off, bytes, 1, blob});
   return off;
@@ -794,6 +839,13 @@ int brax_system_create(const brax_desc* desc, brax_system** out) {
   s->pair_groups = 1;
   s->pair_variant = 0;
   s->pair_mode = (s->paired && 32 * s->B <= pair_variant_max_threads(0)) ? 1 : 0;
+  s->n_limbs = S->n_limbs;
+  for (int b = 0; b < S->B; ++b)
+    s->frozen = s->frozen || (reinterpret_cast<const BodyP*>(s->blob.data() + blob_bodies_off())[b].flags & kAnyFrozen);
+  if (s->n_limbs > 0) {  // the limb layout (its kernels give the paired kernel's bits)
+    s->pair_mode = 1;
+    s->pair_variant = kLimbVariant;
+  }
   *out = s;
   return BRAX_OK;
 }
@@ -839,11 +891,13 @@ int brax_system_set_launch(brax_system* s, int32_t groups, int32_t variant) {
 // Two-environments-per-thread launch override (mode 0: off, 1: on; groups of
 // 64 environments per block; launch-bounds variant); used by the autotuner.
 int brax_system_set_pair_launch(brax_system* s, int32_t mode, int32_t groups, int32_t variant) {
-  if (!s || mode < 0 || mode > 1 || groups < 1 || groups > 15 || variant < 0 || variant > 4)
+  if (!s || mode < 0 || mode > 1 || groups < 1 || groups > 15 || variant < 0 || variant > kLimbSplit)
     return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_system_set_pair_launch: bad arguments");
+  if (mode == 1 && variant >= kLimbVariant && s->n_limbs == 0)
+    return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_system_set_pair_launch: the system has no limb layout");
   if (mode == 1 && !s->paired)
     return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_system_set_pair_launch: the system has no paired kernel");
-  if (mode == 1 && 32 * s->B * groups > pair_variant_max_threads(variant))
+  if (mode == 1 && variant < kLimbVariant && 32 * s->B * groups > pair_variant_max_threads(variant))
     return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_system_set_pair_launch: block too large for the variant");
   s->pair_mode = mode;
   if (mode == 1) {
@@ -944,6 +998,50 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   // is switched on, checkpointing rollouts included: the reverse pass
   // rebuilds a checkpoint segment's step states with the kernel that wrote
   // the checkpoints (rollout_backward_impl), so gradients do not depend on K.
+  if (s->pair_mode == 1 && s->pair_variant >= kLimbVariant) {
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess) {
+      cudaGetLastError();
+      n_sm = 1;
+    }
+    LimbLaunch ll;
+    ll.n_limbs = s->n_limbs;
+    ll.frozen = s->frozen;
+    ll.env = env != nullptr;
+    // The split kernel while its warps (a quarter of the wide kernel's
+    // environments each) are at most 23 an SM, 14,000 quadrupeds: there it
+    // takes 25 us a step and the wide kernel 25.6; beyond, the wide kernel's
+    // warps fill the SMs (measured table at rollout_limb_split_kernel).
+    const int64_t split_warps = (n_envs + limb_warp_envs(s->n_limbs, true) - 1) / limb_warp_envs(s->n_limbs, true);
+    ll.split = s->pair_variant == kLimbVariant ? split_warps <= 23LL * n_sm : s->pair_variant == kLimbSplit;
+    // blocks of one warp until every SM has one, then up to four (one per
+    // scheduler of an SM)
+    const int64_t per_warp = limb_warp_envs(s->n_limbs, ll.split), n_warps = (n_envs + per_warp - 1) / per_warp;
+    ll.warps = (int)std::min<int64_t>(kLimbMaxWarps, (n_warps + n_sm - 1) / n_sm);
+    const int64_t grid = (n_warps + ll.warps - 1) / ll.warps;
+    if (grid > 0x7fffffff) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout: too many environments");
+    Seg sg = make_seg(s, ll.warps, n_envs);
+    sg.cta_begin = 0;
+    sg.cta_end = (int32_t)grid;
+    sg.state0 = state0;
+    sg.actions = actions;
+    sg.state_T = state_T;
+    sg.ckpt = checkpoints;
+    sg.torso = torso_traj;
+    sg.ccount = contact_count;
+    apply_env(s, sg, env);
+    L.seg[0] = sg;
+    const SchedPlan pl =
+        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, limb_blocks_per_sm(ll));
+    int64_t launch_grid;
+    cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
+                                   as_stream(stream), fr);
+    s->last_grid = launch_grid;
+    s->last_chunks = L.sc.n_chunks;
+    s->last_chunk_steps = L.sc.chunk_steps;
+    if (e == cudaSuccess) e = launch_rollout_limb(L, ll, (int)launch_grid, as_stream(stream));
+    return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout");
+  }
   if (s->pair_mode == 1) {
     Seg sg = make_seg(s, s->pair_groups, n_envs);
     const int64_t per_cta = 64LL * s->pair_groups;

@@ -244,78 +244,6 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
 }
 
 // ------------------------------------------------------------------ two environments per thread
-namespace p2 {
-// Load environment A's and B's body into the pair state (a padding half
-// steps the body's rest pose).
-__device__ __forceinline__ void load_pair(const float* pa, const float* pb, const BodyP& bp, Body& s) {
-  auto ld = [&](int i) {
-    const float r = i < 3 ? bp.rest_pos[i] : (i < 7 ? bp.rest_rot[i - 3] : 0.f);
-    return make_float2(pa ? __ldcg(pa + i) : r, pb ? __ldcg(pb + i) : r);
-  };
-  s.x = V{ld(0), ld(1), ld(2)};
-  s.qw = ld(3);
-  s.qx = ld(4);
-  s.qy = ld(5);
-  s.qz = ld(6);
-  s.v = V{ld(7), ld(8), ld(9)};
-  s.w = V{ld(10), ld(11), ld(12)};
-}
-// Store one half (0: A, 1: B) of the pair state.
-__device__ __forceinline__ void store_half(float* p, const Body& s, int half) {
-  auto h = [half](f2 v) { return half ? v.y : v.x; };
-  p[0] = h(s.x.x);
-  p[1] = h(s.x.y);
-  p[2] = h(s.x.z);
-  p[3] = h(s.qw);
-  p[4] = h(s.qx);
-  p[5] = h(s.qy);
-  p[6] = h(s.qz);
-  p[7] = h(s.v.x);
-  p[8] = h(s.v.y);
-  p[9] = h(s.v.z);
-  p[10] = h(s.w.x);
-  p[11] = h(s.w.y);
-  p[12] = h(s.w.z);
-}
-// One environment (half 0: A, 1: B) of the pair state as a scalar body.
-__device__ __forceinline__ brax::Body half_body(const Body& s, int h) {
-  auto c = [h](f2 v) { return h ? v.y : v.x; };
-  brax::Body o;
-  o.x = mk3(c(s.x.x), c(s.x.y), c(s.x.z));
-  o.qw = c(s.qw);
-  o.qx = c(s.qx);
-  o.qy = c(s.qy);
-  o.qz = c(s.qz);
-  o.v = mk3(c(s.v.x), c(s.v.y), c(s.v.z));
-  o.w = mk3(c(s.w.x), c(s.w.y), c(s.w.z));
-  return o;
-}
-// Replace one half of the pair state by the 13 floats at p.
-__device__ __forceinline__ void load_half(const float* p, Body& s, int h) {
-  auto set = [h](f2& v, float x) {
-    if (h) v.y = x;
-    else v.x = x;
-  };
-  set(s.x.x, p[0]);
-  set(s.x.y, p[1]);
-  set(s.x.z, p[2]);
-  set(s.qw, p[3]);
-  set(s.qx, p[4]);
-  set(s.qy, p[5]);
-  set(s.qz, p[6]);
-  set(s.v.x, p[7]);
-  set(s.v.y, p[8]);
-  set(s.v.z, p[9]);
-  set(s.w.x, p[10]);
-  set(s.w.y, p[11]);
-  set(s.w.z, p[12]);
-}
-__device__ __forceinline__ bool finite_pair(const Body& s) {
-  const f2 t = add(add(add(s.x.x, s.x.y), add(s.x.z, s.qw)),
-                   add(add(add(s.qx, s.qy), add(s.qz, s.v.x)), add(add(s.v.y, s.v.z), add(s.w.x, add(s.w.y, s.w.z)))));
-  return fabsf(t.x) < INFINITY && fabsf(t.y) < INFINITY;
-}
-}  // namespace p2
 
 // Persistent rollout of a hinge-only system, two environments per thread
 // (brax_pair.cuh).  A block holds G groups of 64 environments (a unit): unit
@@ -469,7 +397,17 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_pair_kernel(const __grid_c
       group_sync(bar, nthr);
       if (has_parent) {
         const p2::Pub pp = read_pub(gm, bp.parent, lane);
-        joint(q, act_idx >= 0, pp, s, f, act, gm.reactf(b, 0) + lane);
+        const JointOut jo = joint(q, q, act_idx >= 0, pp, s, f.R, act);
+        f2* r = gm.reactf(b, 0) + lane;
+        r[0 * 32] = jo.F_.x;  // the parent takes -F: it subtracts
+        r[1 * 32] = jo.F_.y;
+        r[2 * 32] = jo.F_.z;
+        r[3 * 32] = jo.tp.x;
+        r[4 * 32] = jo.tp.y;
+        r[5 * 32] = jo.tp.z;
+        r[6 * 32] = jo.tc.x;  // the child's own torque (its force is F)
+        r[7 * 32] = jo.tc.y;
+        r[8 * 32] = jo.tc.z;
       }
       {
         const f2* pr = gm.pubf(b, 3) + lane;
@@ -478,12 +416,12 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_pair_kernel(const __grid_c
       }
       p2::Acc acc{vzero(), vzero(), 0, 0};
       f.Ii = inv_inertia_world(f.R, q.inv_I);  // not needed by the joint: computed after it
-      if (kFlat) plane_points_z(S2, q, bp.flags, np, s, f, acc);
+      if (kFlat) plane_points_z(S2, q, q, bp.flags, np, s, f, acc);
       else plane_points(S2, q, bp.flags, np, s, f, acc);
       cca += acc.na;
       ccb += acc.nb;
       group_sync(bar, nthr);
-      integrate(S2, average, bp, q, gm, b, lane, s, f, acc);
+      integrate(S2, average, bp.flags, q, gather_wrench(bp, gm, b, lane), s, f, acc);
     }
     if (sg.torso && b == 0) {
       float* tp = sg.torso + (int64_t)t * N * 3;

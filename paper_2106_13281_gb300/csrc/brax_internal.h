@@ -11,6 +11,10 @@
 #include "../../include/brax.h"
 
 namespace brax {
+// Paired variants of the limb layout: the kernel picked by the number of
+// environments, the wide one (two environments a lane), the split one (one
+// limb body a lane).
+constexpr int kLimbVariant = 5, kLimbWide = 6, kLimbSplit = 7;
 // Scheduler scratch of chunked rollouts: kRing regions of (32 + units) int32,
 // taken in turn by successive launches so that rollouts on different streams
 // do not share one; replaced buffers are freed with the owner.
@@ -40,7 +44,9 @@ struct brax_system {
   bool paired = false;
   int pair_mode = 0;
   int pair_groups = 1;   // groups of 64 environments per thread block
-  int pair_variant = 0;  // launch-bounds variant of the paired kernel
+  int pair_variant = 0;  // launch-bounds variant of the paired kernel, or kLimbVariant
+  bool frozen = false;   // some body has a frozen axis
+  int n_limbs = 0;       // limbs of a system in the limb layout (brax_limb.cuh), else 0
   int bwd_variant = -1;  // launch-bounds variant of the reverse kernel (-1: smallest that fits)
   // Chunked schedule of rollouts (Sched in brax_device.cuh).  Mode 1
   // (default): used when the blocks do not fill a whole number of resident

@@ -26,6 +26,18 @@ int pair_variant_max_threads(int variant);
 // Resident blocks per SM of a paired-kernel variant (0 if it cannot launch).
 int pair_blocks_per_sm(int variant, int threads, size_t smem);
 size_t pair_group_bytes(int B, int A);
+// The limb layout (brax_limb.cuh; systems whose SysP::n_limbs > 0): blocks of
+// 1..kLimbMaxWarps independent warps of limb_warp_envs environments each.
+// split: one limb body a lane instead of one limb of two environments.
+constexpr int kLimbMaxWarps = 4;
+struct LimbLaunch {
+  int n_limbs, warps;
+  bool frozen, split, env;
+};
+inline int limb_warp_envs(int n_limbs, bool split) { return (split ? 16 : 64) / n_limbs; }
+cudaError_t launch_rollout_limb(const Launch& L, const LimbLaunch& l, int grid, cudaStream_t st);
+int limb_blocks_per_sm(const LimbLaunch& l);
+cudaError_t upload_pool_limb(int off, const void* data, size_t bytes);
 // iso: a hinge-only system whose bodies all have isotropic inertia (the
 // two-barrier reverse substep); ignored when general.
 cudaError_t launch_rollout_backward(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,

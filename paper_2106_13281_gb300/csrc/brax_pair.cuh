@@ -21,6 +21,10 @@ namespace p2 {
 
 using f2 = float2;
 
+// Every function of the arithmetic is a template over the number F: f2 (two
+// values a register pair, packed instructions) or float (one value, the same
+// rounding: explicit round-to-nearest multiplies and adds, which the compiler
+// does not fuse), so that kernels of either width give the same bits.
 __device__ __forceinline__ f2 add(f2 a, f2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ f2 mul(f2 a, f2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ f2 fma(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
@@ -35,42 +39,91 @@ __device__ __forceinline__ f2 sub(f2 a, f2 b) {
   memcpy(&d, &rd, 8);
   return d;
 }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ f2 zero2() { return make_float2(0.f, 0.f); }
-__device__ __forceinline__ f2 neg(f2 a) { return sub(zero2(), a); }
+template <class F>
+__device__ __forceinline__ F num(float v);
+template <>
+__device__ __forceinline__ f2 num<f2>(float v) {
+  return make_float2(v, v);
+}
+template <>
+__device__ __forceinline__ float num<float>(float v) {
+  return v;
+}
+template <class F>
+__device__ __forceinline__ F neg(F a) {
+  return sub(num<F>(0.f), a);
+}
 
-struct V {
-  f2 x, y, z;
+template <class F>
+struct VT {
+  F x, y, z;
 };
-__device__ __forceinline__ V vzero() { return V{zero2(), zero2(), zero2()}; }
-__device__ __forceinline__ V vadd(V a, V b) { return V{add(a.x, b.x), add(a.y, b.y), add(a.z, b.z)}; }
-__device__ __forceinline__ V vsub(V a, V b) { return V{sub(a.x, b.x), sub(a.y, b.y), sub(a.z, b.z)}; }
-__device__ __forceinline__ V vscale(f2 s, V a) { return V{mul(s, a.x), mul(s, a.y), mul(s, a.z)}; }
-__device__ __forceinline__ V vfma(f2 s, V a, V b) { return V{fma(s, a.x, b.x), fma(s, a.y, b.y), fma(s, a.z, b.z)}; }
-__device__ __forceinline__ f2 dot(V a, V b) { return fma(a.x, b.x, fma(a.y, b.y, mul(a.z, b.z))); }
-__device__ __forceinline__ V cross(V a, V b) {
-  return V{sub(mul(a.y, b.z), mul(a.z, b.y)), sub(mul(a.z, b.x), mul(a.x, b.z)), sub(mul(a.x, b.y), mul(a.y, b.x))};
+using V = VT<f2>;
+template <class F = f2>
+__device__ __forceinline__ VT<F> vzero() {
+  return VT<F>{num<F>(0.f), num<F>(0.f), num<F>(0.f)};
+}
+template <class F>
+__device__ __forceinline__ VT<F> vadd(VT<F> a, VT<F> b) {
+  return VT<F>{add(a.x, b.x), add(a.y, b.y), add(a.z, b.z)};
+}
+template <class F>
+__device__ __forceinline__ VT<F> vsub(VT<F> a, VT<F> b) {
+  return VT<F>{sub(a.x, b.x), sub(a.y, b.y), sub(a.z, b.z)};
+}
+template <class F>
+__device__ __forceinline__ VT<F> vscale(F s, VT<F> a) {
+  return VT<F>{mul(s, a.x), mul(s, a.y), mul(s, a.z)};
+}
+template <class F>
+__device__ __forceinline__ VT<F> vfma(F s, VT<F> a, VT<F> b) {
+  return VT<F>{fma(s, a.x, b.x), fma(s, a.y, b.y), fma(s, a.z, b.z)};
+}
+template <class F>
+__device__ __forceinline__ F dot(VT<F> a, VT<F> b) {
+  return fma(a.x, b.x, fma(a.y, b.y, mul(a.z, b.z)));
+}
+template <class F>
+__device__ __forceinline__ VT<F> cross(VT<F> a, VT<F> b) {
+  return VT<F>{sub(mul(a.y, b.z), mul(a.z, b.y)), sub(mul(a.z, b.x), mul(a.x, b.z)), sub(mul(a.x, b.y), mul(a.y, b.x))};
 }
 // c + a x b
-__device__ __forceinline__ V cross_add(V a, V b, V c) {
-  return V{sub(fma(a.y, b.z, c.x), mul(a.z, b.y)), sub(fma(a.z, b.x, c.y), mul(a.x, b.z)),
-           sub(fma(a.x, b.y, c.z), mul(a.y, b.x))};
+template <class F>
+__device__ __forceinline__ VT<F> cross_add(VT<F> a, VT<F> b, VT<F> c) {
+  return VT<F>{sub(fma(a.y, b.z, c.x), mul(a.z, b.y)), sub(fma(a.z, b.x, c.y), mul(a.x, b.z)),
+               sub(fma(a.x, b.y, c.z), mul(a.y, b.x))};
 }
-__device__ __forceinline__ V vld(const f2* p) { return V{p[0], p[1], p[2]}; }
+template <class F>
+__device__ __forceinline__ VT<F> vld(const F* p) {
+  return VT<F>{p[0], p[1], p[2]};
+}
 
-struct M {
-  f2 m[9];
+template <class F>
+struct MT {
+  F m[9];
 };
-__device__ __forceinline__ V mulv(const M& R, V o) {
-  return V{fma(R.m[0], o.x, fma(R.m[1], o.y, mul(R.m[2], o.z))), fma(R.m[3], o.x, fma(R.m[4], o.y, mul(R.m[5], o.z))),
-           fma(R.m[6], o.x, fma(R.m[7], o.y, mul(R.m[8], o.z)))};
+using M = MT<f2>;
+template <class F>
+__device__ __forceinline__ VT<F> mulv(const MT<F>& R, VT<F> o) {
+  return VT<F>{fma(R.m[0], o.x, fma(R.m[1], o.y, mul(R.m[2], o.z))), fma(R.m[3], o.x, fma(R.m[4], o.y, mul(R.m[5], o.z))),
+               fma(R.m[6], o.x, fma(R.m[7], o.y, mul(R.m[8], o.z)))};
 }
-__device__ __forceinline__ V mulc(const M& R, const f2* o) { return mulv(R, vld(o)); }
+template <class F>
+__device__ __forceinline__ VT<F> mulc(const MT<F>& R, const F* o) {
+  return mulv(R, vld(o));
+}
 
-__device__ __forceinline__ M qmat(f2 qw, f2 qx, f2 qy, f2 qz, f2 one) {
-  const f2 x2 = add(qx, qx), y2 = add(qy, qy), z2 = add(qz, qz);
-  const f2 xx = mul(qx, x2), yy = mul(qy, y2), zz = mul(qz, z2);
-  const f2 wx = mul(qw, x2), wy = mul(qw, y2), wz = mul(qw, z2);
-  M R;
+template <class F>
+__device__ __forceinline__ MT<F> qmat(F qw, F qx, F qy, F qz, F one) {
+  const F x2 = add(qx, qx), y2 = add(qy, qy), z2 = add(qz, qz);
+  const F xx = mul(qx, x2), yy = mul(qy, y2), zz = mul(qz, z2);
+  const F wx = mul(qw, x2), wy = mul(qw, y2), wz = mul(qw, z2);
+  MT<F> R;
   R.m[0] = sub(sub(one, yy), zz);
   R.m[1] = sub(mul(qx, y2), wz);
   R.m[2] = fma(qx, z2, wy);
@@ -84,49 +137,77 @@ __device__ __forceinline__ M qmat(f2 qw, f2 qx, f2 qy, f2 qz, f2 one) {
 }
 
 // Symmetric world inverse inertia R diag(d) R^T (xx, xy, xz, yy, yz, zz).
-struct S6 {
-  f2 a[6];
+template <class F>
+struct S6T {
+  F a[6];
 };
-__device__ __forceinline__ S6 inv_inertia_world(const M& R, const f2* d) {
-  S6 s;
-  const f2 r00 = mul(R.m[0], d[0]), r01 = mul(R.m[1], d[1]), r02 = mul(R.m[2], d[2]);
-  const f2 r10 = mul(R.m[3], d[0]), r11 = mul(R.m[4], d[1]), r12 = mul(R.m[5], d[2]);
+using S6 = S6T<f2>;
+template <class F>
+__device__ __forceinline__ S6T<F> inv_inertia_world(const MT<F>& R, const F* d) {
+  S6T<F> s;
+  const F r00 = mul(R.m[0], d[0]), r01 = mul(R.m[1], d[1]), r02 = mul(R.m[2], d[2]);
+  const F r10 = mul(R.m[3], d[0]), r11 = mul(R.m[4], d[1]), r12 = mul(R.m[5], d[2]);
   s.a[0] = fma(r00, R.m[0], fma(r01, R.m[1], mul(r02, R.m[2])));
   s.a[1] = fma(r00, R.m[3], fma(r01, R.m[4], mul(r02, R.m[5])));
   s.a[2] = fma(r00, R.m[6], fma(r01, R.m[7], mul(r02, R.m[8])));
   s.a[3] = fma(r10, R.m[3], fma(r11, R.m[4], mul(r12, R.m[5])));
   s.a[4] = fma(r10, R.m[6], fma(r11, R.m[7], mul(r12, R.m[8])));
-  const f2 r20 = mul(R.m[6], d[0]), r21 = mul(R.m[7], d[1]), r22 = mul(R.m[8], d[2]);
+  const F r20 = mul(R.m[6], d[0]), r21 = mul(R.m[7], d[1]), r22 = mul(R.m[8], d[2]);
   s.a[5] = fma(r20, R.m[6], fma(r21, R.m[7], mul(r22, R.m[8])));
   return s;
 }
-__device__ __forceinline__ V mul6(const S6& s, V v) {
-  return V{fma(s.a[0], v.x, fma(s.a[1], v.y, mul(s.a[2], v.z))), fma(s.a[1], v.x, fma(s.a[3], v.y, mul(s.a[4], v.z))),
-           fma(s.a[2], v.x, fma(s.a[4], v.y, mul(s.a[5], v.z)))};
+template <class F>
+__device__ __forceinline__ VT<F> mul6(const S6T<F>& s, VT<F> v) {
+  return VT<F>{fma(s.a[0], v.x, fma(s.a[1], v.y, mul(s.a[2], v.z))), fma(s.a[1], v.x, fma(s.a[3], v.y, mul(s.a[4], v.z))),
+               fma(s.a[2], v.x, fma(s.a[4], v.y, mul(s.a[5], v.z)))};
 }
 
-__device__ __forceinline__ V mask(uint32_t bits, V a) {
-  return V{(bits & 1u) ? zero2() : a.x, (bits & 2u) ? zero2() : a.y, (bits & 4u) ? zero2() : a.z};
+template <class F>
+__device__ __forceinline__ VT<F> mask(uint32_t bits, VT<F> a) {
+  const F z = num<F>(0.f);
+  return VT<F>{(bits & 1u) ? z : a.x, (bits & 2u) ? z : a.y, (bits & 4u) ? z : a.z};
+}
+
+// Frozen axes: one set of body flags for both values, or one for each.
+struct Flags2 {
+  uint32_t a, b;
+};
+__device__ __forceinline__ bool frozen(uint32_t f) { return (f & kAnyFrozen) != 0; }
+__device__ __forceinline__ bool frozen(Flags2 f) { return ((f.a | f.b) & kAnyFrozen) != 0; }
+__device__ __forceinline__ uint32_t rot_bits(uint32_t f) { return f >> 3; }
+__device__ __forceinline__ Flags2 rot_bits(Flags2 f) { return Flags2{f.a >> 3, f.b >> 3}; }
+// Axis i of `bits` frozen: zero in place of a.
+template <class F>
+__device__ __forceinline__ F mask1(uint32_t bits, int i, F a) {
+  return (bits >> i) & 1u ? num<F>(0.f) : a;
+}
+__device__ __forceinline__ f2 mask1(Flags2 bits, int i, f2 a) {
+  return make_float2((bits.a >> i) & 1u ? 0.f : a.x, (bits.b >> i) & 1u ? 0.f : a.y);
+}
+__device__ __forceinline__ V mask(Flags2 bits, V a) {
+  return V{mask1(bits, 0, a.x), mask1(bits, 1, a.y), mask1(bits, 2, a.z)};
 }
 
 // Per-environment arctangent (the scalar kernel's fast_atan2: octant
 // reduction, the same degree-7 polynomial, octant undone), with the
 // polynomial evaluated packed.
+template <class F>
+__device__ __forceinline__ F atan_poly(F s) {
+  F p = num<F>(-0.004037295f);
+  p = fma(p, s, num<F>(0.021790044f));
+  p = fma(p, s, num<F>(-0.055787466f));
+  p = fma(p, s, num<F>(0.096311055f));
+  p = fma(p, s, num<F>(-0.13903217f));
+  p = fma(p, s, num<F>(0.19945158f));
+  p = fma(p, s, num<F>(-0.3332969f));
+  return fma(p, s, num<F>(0.9999993f));
+}
 __device__ __forceinline__ f2 atan2p(f2 y, f2 x) {
   const float axa = fabsf(x.x), aya = fabsf(y.x), axb = fabsf(x.y), ayb = fabsf(y.y);
   const float mxa = fmaxf(axa, aya), mna = fminf(axa, aya);
   const float mxb = fmaxf(axb, ayb), mnb = fminf(axb, ayb);
   const f2 a = make_float2(mxa > 0.f ? __fdividef(mna, mxa) : 0.f, mxb > 0.f ? __fdividef(mnb, mxb) : 0.f);
-  const f2 s = mul(a, a);
-  f2 p = make_float2(-0.004037295f, -0.004037295f);
-  p = fma(p, s, make_float2(0.021790044f, 0.021790044f));
-  p = fma(p, s, make_float2(-0.055787466f, -0.055787466f));
-  p = fma(p, s, make_float2(0.096311055f, 0.096311055f));
-  p = fma(p, s, make_float2(-0.13903217f, -0.13903217f));
-  p = fma(p, s, make_float2(0.19945158f, 0.19945158f));
-  p = fma(p, s, make_float2(-0.3332969f, -0.3332969f));
-  p = fma(p, s, make_float2(0.9999993f, 0.9999993f));
-  const f2 r = mul(a, p);
+  const f2 r = mul(a, atan_poly(mul(a, a)));
   float ra = r.x, rb = r.y;
   if (aya > axa) ra = 1.5707963267948966f - ra;
   if (ayb > axb) rb = 1.5707963267948966f - rb;
@@ -134,16 +215,38 @@ __device__ __forceinline__ f2 atan2p(f2 y, f2 x) {
   if (x.y < 0.f) rb = 3.141592653589793f - rb;
   return make_float2(copysignf(ra, y.x), copysignf(rb, y.y));
 }
+__device__ __forceinline__ float atan2p(float y, float x) {
+  const float ax = fabsf(x), ay = fabsf(y);
+  const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
+  const float a = mx > 0.f ? __fdividef(mn, mx) : 0.f;
+  float r = mul(a, atan_poly(mul(a, a)));
+  if (ay > ax) r = 1.5707963267948966f - r;
+  if (x < 0.f) r = 3.141592653589793f - r;
+  return copysignf(r, y);
+}
+// Deflection beyond a one-sided limit, given lo - th and hi - th.
+__device__ __forceinline__ float deflection(float th, float lo, float hi, float dlo, float dhi) {
+  return th < lo ? dlo : (th > hi ? dhi : 0.f);
+}
+__device__ __forceinline__ f2 deflection(f2 th, f2 lo, f2 hi, f2 dlo, f2 dhi) {
+  return make_float2(deflection(th.x, lo.x, hi.x, dlo.x, dhi.x), deflection(th.y, lo.y, hi.y, dlo.y, dhi.y));
+}
+__device__ __forceinline__ float clamp_act(float a) { return fminf(fmaxf(a, -1.f), 1.f); }
+__device__ __forceinline__ f2 clamp_act(f2 a) { return make_float2(clamp_act(a.x), clamp_act(a.y)); }
 
-struct Body {
-  V x;
-  f2 qw, qx, qy, qz;
-  V v, w;
+template <class F>
+struct BodyT {
+  VT<F> x;
+  F qw, qx, qy, qz;
+  VT<F> v, w;
 };
-struct Frame {
-  M R;
-  S6 Ii;
+using Body = BodyT<f2>;
+template <class F>
+struct FrameT {
+  MT<F> R;
+  S6T<F> Ii;
 };
+using Frame = FrameT<f2>;
 struct Acc {
   V dv, dw;
   int na, nb;  // active contacts of environment A and B
@@ -241,23 +344,29 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* m, uint32_t parity, int64_t 
 }
 
 // ------------------------------------------------------------------ phase K
+__device__ __forceinline__ float rsqrt_each(float a) { return rsqrtf(a); }
+__device__ __forceinline__ f2 rsqrt_each(f2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+// The integration itself, velocities masked already.
+template <class F>
+__device__ __forceinline__ void advance(F h, F mhh, F hh, BodyT<F>& s) {
+  s.x = vfma(h, s.v, s.x);
+  const F nw = fma(mhh, fma(s.w.x, s.qx, fma(s.w.y, s.qy, mul(s.w.z, s.qz))), s.qw);
+  const F nx = fma(hh, sub(fma(s.qw, s.w.x, mul(s.w.y, s.qz)), mul(s.w.z, s.qy)), s.qx);
+  const F ny = fma(hh, sub(fma(s.qw, s.w.y, mul(s.w.z, s.qx)), mul(s.w.x, s.qz)), s.qy);
+  const F nz = fma(hh, sub(fma(s.qw, s.w.z, mul(s.w.x, s.qy)), mul(s.w.y, s.qx)), s.qz);
+  const F n2 = fma(nw, nw, fma(nx, nx, fma(ny, ny, mul(nz, nz))));
+  const F inv = rsqrt_each(n2);
+  s.qw = mul(nw, inv);
+  s.qx = mul(nx, inv);
+  s.qy = mul(ny, inv);
+  s.qz = mul(nz, inv);
+}
 __device__ __forceinline__ void kinematic(const SysP2& S2, uint32_t flags, Body& s) {
   if (flags & kAnyFrozen) {
     s.v = mask(flags, s.v);
     s.w = mask(flags >> 3, s.w);
   }
-  s.x = vfma(S2.h, s.v, s.x);
-  const f2 hh = S2.hh;
-  const f2 nw = fma(S2.mhh, fma(s.w.x, s.qx, fma(s.w.y, s.qy, mul(s.w.z, s.qz))), s.qw);
-  const f2 nx = fma(hh, sub(fma(s.qw, s.w.x, mul(s.w.y, s.qz)), mul(s.w.z, s.qy)), s.qx);
-  const f2 ny = fma(hh, sub(fma(s.qw, s.w.y, mul(s.w.z, s.qx)), mul(s.w.x, s.qz)), s.qy);
-  const f2 nz = fma(hh, sub(fma(s.qw, s.w.z, mul(s.w.x, s.qy)), mul(s.w.y, s.qx)), s.qz);
-  const f2 n2 = fma(nw, nw, fma(nx, nx, fma(ny, ny, mul(nz, nz))));
-  const f2 inv = make_float2(rsqrtf(n2.x), rsqrtf(n2.y));
-  s.qw = mul(nw, inv);
-  s.qx = mul(nx, inv);
-  s.qy = mul(ny, inv);
-  s.qz = mul(nz, inv);
+  advance(S2.h, S2.mhh, S2.hh, s);
 }
 
 __device__ __forceinline__ void publish(GroupMem2& gm, int b, int lane, const Body& s, const Frame& f) {
@@ -274,11 +383,13 @@ __device__ __forceinline__ void publish(GroupMem2& gm, int b, int lane, const Bo
   p[16 * 32] = s.w.y;
   p[17 * 32] = s.w.z;
 }
-struct Pub {
-  V x;
-  M R;
-  V v, w;
+template <class F>
+struct PubT {
+  VT<F> x;
+  MT<F> R;
+  VT<F> v, w;
 };
+using Pub = PubT<f2>;
 __device__ __forceinline__ Pub read_pub(GroupMem2& gm, int b, int lane) {
   const f2* p = gm.pubf(b, 0) + lane;
   Pub o;
@@ -293,58 +404,54 @@ __device__ __forceinline__ Pub read_pub(GroupMem2& gm, int b, int lane) {
 // ------------------------------------------------------------------ phase J: hinge joint
 // The scalar kernel's hinge (Sec. 3 joint.revolute, Sec. 7.1, App. A limits,
 // torque actuator); returns the child's wrench and writes the parent's.
+// q gives the scalars (stiffnesses, limits, gear), g the geometry (offsets
+// and joint frames): one BodyP2 for both, or a limb's own geometry.
 struct Wrench {
   V F, tau;
 };
-__device__ __forceinline__ Wrench joint(const BodyP2& q, bool has_act, const Pub& pp, const Body& s, const Frame& f,
-                                        f2 act, f2* react_out) {
-  const V rp = mulc(pp.R, q.off_p);
-  const V rc = mulc(f.R, q.off_c);
+template <class F>
+struct JointOutT {
+  VT<F> F_, tc, tp;  // force on the child (the parent takes -F_), torque on the child, torque on the parent
+};
+using JointOut = JointOutT<f2>;
+template <class F, class Par, class Geo>
+__device__ __forceinline__ JointOutT<F> joint(const Par& q, const Geo& g, bool has_act, const PubT<F>& pp,
+                                              const BodyT<F>& s, const MT<F>& R, F act) {
+  using V = VT<F>;
+  const V rp = mulc(pp.R, g.off_p);
+  const V rc = mulc(R, g.off_c);
   const V dpc = vsub(vadd(pp.x, rp), vadd(s.x, rc));
   const V up = cross_add(pp.w, rp, pp.v);
   const V uc = cross_add(s.w, rc, s.v);
   const V du = vsub(uc, up);
-  const V F = V{fma(q.k, dpc.x, mul(q.mc, du.x)), fma(q.k, dpc.y, mul(q.mc, du.y)), fma(q.k, dpc.z, mul(q.mc, du.z))};
-  V tc = cross(rc, F);
-  V tp = cross(F, rp);
-  const V P0 = mulc(pp.R, q.ap + 0);
-  const V P1 = mulc(pp.R, q.ap + 3);
+  const V Fo = V{fma(q.k, dpc.x, mul(q.mc, du.x)), fma(q.k, dpc.y, mul(q.mc, du.y)), fma(q.k, dpc.z, mul(q.mc, du.z))};
+  V tc = cross(rc, Fo);
+  V tp = cross(Fo, rp);
+  const V P0 = mulc(pp.R, g.ap + 0);
+  const V P1 = mulc(pp.R, g.ap + 3);
   const V wr = vsub(s.w, pp.w);
-  const V Ac = mulc(f.R, q.ac + 0);
-  const V yc = mulc(f.R, q.ac + 3);
-  const f2 th = atan2p(dot(cross(P1, yc), P0), dot(P1, yc));
+  const V Ac = mulc(R, g.ac + 0);
+  const V yc = mulc(R, g.ac + 3);
+  const F th = atan2p(dot(cross(P1, yc), P0), dot(P1, yc));
   // one-sided limit springs, per environment
-  const f2 dlo = sub(q.lo, th), dhi = sub(q.hi, th);
-  const f2 Ld = make_float2(th.x < q.lo.x ? dlo.x : (th.x > q.hi.x ? dhi.x : 0.f),
-                            th.y < q.lo.y ? dlo.y : (th.y > q.hi.y ? dhi.y : 0.f));
-  f2 sc = fma(q.kl, Ld, mul(q.mca, dot(wr, P0)));
-  if (has_act) {
-    const f2 a = make_float2(fminf(fmaxf(act.x, -1.f), 1.f), fminf(fmaxf(act.y, -1.f), 1.f));
-    sc = fma(q.gear, a, sc);
-  }
+  const F Ld = deflection(th, q.lo, q.hi, sub(q.lo, th), sub(q.hi, th));
+  F sc = fma(q.kl, Ld, mul(q.mca, dot(wr, P0)));
+  if (has_act) sc = fma(q.gear, clamp_act(act), sc);
   const V tj = vfma(sc, P0, vscale(q.ka, cross(Ac, P0)));
   tc = vadd(tc, tj);
   tp = vsub(tp, tj);
-  react_out[0 * 32] = F.x;  // the parent takes -F: it subtracts
-  react_out[1 * 32] = F.y;
-  react_out[2 * 32] = F.z;
-  react_out[3 * 32] = tp.x;
-  react_out[4 * 32] = tp.y;
-  react_out[5 * 32] = tp.z;
-  react_out[6 * 32] = tc.x;  // the child's own torque (its force is F)
-  react_out[7 * 32] = tc.y;
-  react_out[8 * 32] = tc.z;
-  return Wrench{F, tc};
+  return JointOutT<F>{Fo, tc, tp};
 }
 
 // ------------------------------------------------------------------ phase J: plane contacts
-__device__ __forceinline__ f2 eff_mass(uint32_t flags, f2 inv_m, const S6& Ii, V l, V dir) {
+template <class Fl>
+__device__ __forceinline__ f2 eff_mass(Fl flags, f2 inv_m, const S6& Ii, V l, V dir) {
   V dm = dir;
   const V ld = cross(l, dir);
   V om = mul6(Ii, ld);
-  if (flags & kAnyFrozen) {
+  if (frozen(flags)) {
     dm = mask(flags, dm);
-    om = mask(flags >> 3, om);
+    om = mask(rot_bits(flags), om);
   }
   return fma(dot(dm, dir), inv_m, dot(om, ld));
 }
@@ -428,19 +535,21 @@ __device__ __forceinline__ void plane_points(const SysP2& S2, const BodyP2& q, u
 // with the products by n's zero components dropped (they contribute exact
 // zeros): l x n = (l.y, -l.x, 0), u_n = u.z, the tangential velocity is
 // (u.x, u.y, 0) and the normal impulse acts along z alone.
-__device__ __forceinline__ void point_response_z(const SysP2& S2, uint32_t flags, f2 inv_m, const PointP2& pt, V l,
-                                                 f2 depth, bool ma, bool mb, const Body& s, const Frame& f,
-                                                 Acc& acc) {
+// kVote: skip the friction when no environment of the warp slides.
+template <bool kVote = true, class Fl, class Pt>
+__device__ __forceinline__ void point_response_z(const SysP2& S2, Fl flags, f2 inv_m, const Pt& pt, V l, f2 depth,
+                                                 bool ma, bool mb, const Body& s, const Frame& f, Acc& acc) {
   const V u = cross_add(s.w, l, s.v);
   // k_n: linear term (unless z is frozen) + (I_w^-1 (l x n)) . (l x n)
   const f2 nlx = neg(l.x);
   f2 omx = fma(f.Ii.a[0], l.y, mul(f.Ii.a[1], nlx));
   f2 omy = fma(f.Ii.a[1], l.y, mul(f.Ii.a[3], nlx));
-  if (flags & kAnyFrozen) {
-    if (flags & (kFrozenRot0 << 0)) omx = zero2();
-    if (flags & (kFrozenRot0 << 1)) omy = zero2();
+  f2 lin = inv_m;
+  if (frozen(flags)) {
+    omx = mask1(rot_bits(flags), 0, omx);
+    omy = mask1(rot_bits(flags), 1, omy);
+    lin = mask1(flags, 2, lin);
   }
-  const f2 lin = (flags & (kFrozenPos0 << 2)) ? zero2() : inv_m;
   const f2 kn = add(lin, fma(omx, l.y, mul(omy, nlx)));
   const bool ka = kn.x > 0.f, kb = kn.y > 0.f;
   ma = ma && ka;
@@ -454,7 +563,7 @@ __device__ __forceinline__ void point_response_z(const SysP2& S2, uint32_t flags
   V J = V{zero2(), zero2(), jn};
   const f2 ut2 = fma(u.x, u.x, mul(u.y, u.y));
   const bool fa = ut2.x > S2.eps2.x, fb = ut2.y > S2.eps2.y;
-  if (__any_sync(0xffffffffu, fa || fb)) {
+  if (!kVote || __any_sync(0xffffffffu, fa || fb)) {
     const f2 rinv = make_float2(fa ? rsqrtf(ut2.x) : 0.f, fb ? rsqrtf(ut2.y) : 0.f);
     const f2 utn = mul(ut2, rinv);
     const V t = V{mul(rinv, u.x), mul(rinv, u.y), zero2()};
@@ -468,9 +577,9 @@ __device__ __forceinline__ void point_response_z(const SysP2& S2, uint32_t flags
   }
   V dv = vscale(inv_m, J);
   V dw = mul6(f.Ii, cross(l, J));
-  if (flags & kAnyFrozen) {
+  if (frozen(flags)) {
     dv = mask(flags, dv);
-    dw = mask(flags >> 3, dw);
+    dw = mask(rot_bits(flags), dw);
   }
   const f2 m = make_float2(ma ? 1.f : 0.f, mb ? 1.f : 0.f);
   acc.dv = vfma(m, dv, acc.dv);
@@ -481,17 +590,18 @@ __device__ __forceinline__ void point_response_z(const SysP2& S2, uint32_t flags
 
 // plane_points for z-up planes: depth r - ((x + R o).z - p0.z), lever
 // R o - r n = (R o).xy, (R o).z - r.
-__device__ __forceinline__ void plane_points_z(const SysP2& S2, const BodyP2& q, uint32_t flags, int np,
+template <class Geo>
+__device__ __forceinline__ void plane_points_z(const SysP2& S2, const BodyP2& q, const Geo& g, uint32_t flags, int np,
                                                const Body& s, const Frame& f, Acc& acc) {
   V l0, l1;
   f2 d0 = make_float2(-1.f, -1.f), d1 = make_float2(-1.f, -1.f);
   if (np > 0) {
-    const V ro = mulc(f.R, q.pt[0].o);
+    const V ro = mulc(f.R, g.point(0));
     d0 = sub(q.pt[0].r, sub(add(s.x.z, ro.z), q.pt[0].p0[2]));
     l0 = V{ro.x, ro.y, add(ro.z, q.pt[0].mr)};
   }
   if (np > 1) {
-    const V ro = mulc(f.R, q.pt[1].o);
+    const V ro = mulc(f.R, g.point(1));
     d1 = sub(q.pt[1].r, sub(add(s.x.z, ro.z), q.pt[1].p0[2]));
     l1 = V{ro.x, ro.y, add(ro.z, q.pt[1].mr)};
   }
@@ -506,10 +616,11 @@ __device__ __forceinline__ void plane_points_z(const SysP2& S2, const BodyP2& q,
 }
 
 // ------------------------------------------------------------------ phase P
-__device__ __forceinline__ void integrate(const SysP2& S2, bool average, const BodyP& bp, const BodyP2& q,
-                                          GroupMem2& gm, int b, int lane, Body& s, const Frame& f, const Acc& acc) {
+// The wrench of a body: its own joint's (parked in shared memory between the
+// joint and here) and its children's reactions, in child order.
+__device__ __forceinline__ Wrench gather_wrench(const BodyP& bp, GroupMem2& gm, int b, int lane) {
   Wrench wr{vzero(), vzero()};
-  if (bp.flags & kHasParent) {  // the own joint's wrench, parked by joint()
+  if (bp.flags & kHasParent) {
     const f2* r = gm.reactf(b, 0) + lane;
     wr.F = V{r[0], r[32], r[64]};
     wr.tau = V{r[6 * 32], r[7 * 32], r[8 * 32]};
@@ -519,12 +630,16 @@ __device__ __forceinline__ void integrate(const SysP2& S2, bool average, const B
     wr.F = vsub(wr.F, V{r[0], r[32], r[64]});
     wr.tau = vadd(wr.tau, V{r[96], r[128], r[160]});
   }
+  return wr;
+}
+__device__ __forceinline__ void integrate(const SysP2& S2, bool average, uint32_t flags, const BodyP2& q,
+                                          const Wrench& wr, Body& s, const Frame& f, const Acc& acc) {
   const f2 h = S2.h;
   V v = vfma(h, vfma(q.inv_mass, wr.F, vld(S2.g)), s.v);
   V w = vfma(h, mul6(f.Ii, wr.tau), s.w);
-  if (bp.flags & kAnyFrozen) {
-    v = mask(bp.flags, v);
-    w = mask(bp.flags >> 3, w);
+  if (flags & kAnyFrozen) {
+    v = mask(flags, v);
+    w = mask(flags >> 3, w);
   }
   // mean (or sum) of the contact velocity changes; a body without contacts
   // adds its zero accumulator
@@ -535,5 +650,76 @@ __device__ __forceinline__ void integrate(const SysP2& S2, bool average, const B
   s.w = vfma(inv, acc.dw, w);
 }
 
+// ------------------------------------------------------------------ state I/O
+// Load environment A's and B's body into the pair state (a padding half
+// steps the body's rest pose).
+__device__ __forceinline__ void load_pair(const float* pa, const float* pb, const BodyP& bp, Body& s) {
+  auto ld = [&](int i) {
+    const float r = i < 3 ? bp.rest_pos[i] : (i < 7 ? bp.rest_rot[i - 3] : 0.f);
+    return make_float2(pa ? __ldcg(pa + i) : r, pb ? __ldcg(pb + i) : r);
+  };
+  s.x = V{ld(0), ld(1), ld(2)};
+  s.qw = ld(3);
+  s.qx = ld(4);
+  s.qy = ld(5);
+  s.qz = ld(6);
+  s.v = V{ld(7), ld(8), ld(9)};
+  s.w = V{ld(10), ld(11), ld(12)};
+}
+// Store one half (0: A, 1: B) of the pair state.
+__device__ __forceinline__ void store_half(float* p, const Body& s, int half) {
+  auto h = [half](f2 v) { return half ? v.y : v.x; };
+  p[0] = h(s.x.x);
+  p[1] = h(s.x.y);
+  p[2] = h(s.x.z);
+  p[3] = h(s.qw);
+  p[4] = h(s.qx);
+  p[5] = h(s.qy);
+  p[6] = h(s.qz);
+  p[7] = h(s.v.x);
+  p[8] = h(s.v.y);
+  p[9] = h(s.v.z);
+  p[10] = h(s.w.x);
+  p[11] = h(s.w.y);
+  p[12] = h(s.w.z);
+}
+// One environment (half 0: A, 1: B) of the pair state as a scalar body.
+__device__ __forceinline__ brax::Body half_body(const Body& s, int h) {
+  auto c = [h](f2 v) { return h ? v.y : v.x; };
+  brax::Body o;
+  o.x = mk3(c(s.x.x), c(s.x.y), c(s.x.z));
+  o.qw = c(s.qw);
+  o.qx = c(s.qx);
+  o.qy = c(s.qy);
+  o.qz = c(s.qz);
+  o.v = mk3(c(s.v.x), c(s.v.y), c(s.v.z));
+  o.w = mk3(c(s.w.x), c(s.w.y), c(s.w.z));
+  return o;
+}
+// Replace one half of the pair state by the 13 floats at p.
+__device__ __forceinline__ void load_half(const float* p, Body& s, int h) {
+  auto set = [h](f2& v, float x) {
+    if (h) v.y = x;
+    else v.x = x;
+  };
+  set(s.x.x, p[0]);
+  set(s.x.y, p[1]);
+  set(s.x.z, p[2]);
+  set(s.qw, p[3]);
+  set(s.qx, p[4]);
+  set(s.qy, p[5]);
+  set(s.qz, p[6]);
+  set(s.v.x, p[7]);
+  set(s.v.y, p[8]);
+  set(s.v.z, p[9]);
+  set(s.w.x, p[10]);
+  set(s.w.y, p[11]);
+  set(s.w.z, p[12]);
+}
+__device__ __forceinline__ bool finite_pair(const Body& s) {
+  const f2 t = add(add(add(s.x.x, s.x.y), add(s.x.z, s.qw)),
+                   add(add(add(s.qx, s.qy), add(s.qz, s.v.x)), add(add(s.v.y, s.v.z), add(s.w.x, add(s.w.y, s.w.z)))));
+  return fabsf(t.x) < INFINITY && fabsf(t.y) < INFINITY;
+}
 }  // namespace p2
 }  // namespace brax

@@ -121,6 +121,10 @@ struct SysP {
   int32_t gyro;       // 1: the potential integrator adds the gyroscopic torque -w x (I_w w)
   int32_t variants;   // 1: damping, gyroscopic term or target-angle actuators (general kernel only)
   int32_t iso;        // 1: every body's inertia is isotropic (I_w = I for every orientation)
+  // Limb layout (brax_limb.cuh): n_limbs > 0 when the system is one root with
+  // n_limbs limbs of two hinged bodies each, alike up to their geometry.
+  int32_t n_limbs, limb_root;
+  int32_t limb_upper[BRAX_MAX_CHILDREN], limb_lower[BRAX_MAX_CHILDREN];  // in the order of the root's children
 };
 
 // Two environments per thread (systems with hinge joints only and at most
@@ -146,6 +150,7 @@ struct BodyP2 {
   float2 k, mc, ka, mca, kl, lo, hi, gear;  // mc = -c, mca = -ca
   float2 inv_mass, inv_I[3];
   PointP2 pt[2];
+  __host__ __device__ const float2* point(int i) const { return pt[i].o; }
 };
 
 // Byte offsets inside the blob.

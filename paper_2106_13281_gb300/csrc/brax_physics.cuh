@@ -686,8 +686,8 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
 // angles, measured as the limits measure them, and the relative angular
 // velocity w - w_p along its world axes R_p (parent joint-frame axis k).
 // Rp, wp: the parent's rotation and angular velocity; R, w: this body's.
-template <bool kGeneral>
-__device__ __forceinline__ void joint_obs(const BodyP& bp, const M3& Rp, V3 wp, const M3& R, V3 w, float* ang,
+template <bool kGeneral, class JP>
+__device__ __forceinline__ void joint_obs(const JP& bp, const M3& Rp, V3 wp, const M3& R, V3 w, float* ang,
                                           float* rate) {
   const V3 P0 = mulc(Rp, bp.ap + 0);
   const V3 P1 = mulc(Rp, bp.ap + 3);

@@ -100,6 +100,7 @@ extern "C" int brax_autotune(brax_system* s, int64_t n_envs, int32_t T, const fl
     if (s->paired)
       for (int v : {0, 3, 1, 4, 2})
         for (int g = 1; g <= 4 && 32 * s->B * g <= brax::pair_variant_max_threads(v); ++g) cands.push_back({1, g, v});
+    if (s->n_limbs > 0) cands.push_back({1, 1, brax::kLimbVariant});
     // the fastest one-environment configuration is kept in any case: it runs
     // the rollouts that write checkpoints
     float best[2] = {-1.f, -1.f};

@@ -189,5 +189,7 @@ def _ptr(t):
 
 def _stream(stream=None):
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the raw handle of the current device's current stream, without building a Stream object (2.9 us)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())

@@ -683,7 +683,7 @@ static BwdKernel bwd_kernel(int variant, bool general, bool iso) {
 
 int backward_blocks_per_sm(int variant, bool general, bool iso, int threads, size_t smem) {
   const BwdKernel k = bwd_kernel(variant, general, iso);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
   return n;
@@ -697,7 +697,7 @@ int backward_variant_max_threads(int variant) {
 cudaError_t launch_rollout_backward(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,
                                     bool iso, cudaStream_t st) {
   const BwdKernel k = bwd_kernel(variant, general, iso);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, threads, smem, st>>>(L);
   return cudaGetLastError();

@@ -702,14 +702,21 @@ SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t
   p.chunk_steps = (int)steps;
   return p;
 }
-SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, int per_sm, int min_chunk = 16) {
-  if (mode == 0 || T < 2 || units < 1 || per_sm < 1) return SchedPlan{};
+// per_sm() gives the resident blocks per SM.  It asks the driver (a microsecond
+// or more, of the ten that a one-step call takes), so only a launch that could
+// be cut asks: not a single step, nor a launch of at most one block an SM.
+template <class PerSm>
+SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, PerSm per_sm, int min_chunk = 16) {
+  if (mode == 0 || T < 2 || units < 1) return SchedPlan{};
   int n_sm = 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
     return SchedPlan{};
   }
-  return plan_schedule_slots(mode, chunk, units, T, (int64_t)per_sm * n_sm, min_chunk);
+  if (mode == 1 && (units <= n_sm || T < 2 * min_chunk)) return SchedPlan{};
+  const int blocks = per_sm();
+  if (blocks < 1) return SchedPlan{};
+  return plan_schedule_slots(mode, chunk, units, T, (int64_t)blocks * n_sm, min_chunk);
 }
 
 // One region of a scheduler scratch for a launch of `units` units (null when
@@ -1032,7 +1039,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     apply_env(s, sg, env);
     L.seg[0] = sg;
     const SchedPlan pl =
-        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, limb_blocks_per_sm(ll));
+        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, [&] { return limb_blocks_per_sm(ll); });
     int64_t launch_grid;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                    as_stream(stream), fr);
@@ -1072,7 +1079,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     }
     const int threads = 32 * s->B * s->pair_groups;
     const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
-                                       pair_blocks_per_sm(s->pair_variant, threads, smem));
+                                       [&] { return pair_blocks_per_sm(s->pair_variant, threads, smem); });
     int64_t launch_grid;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                    as_stream(stream), fr);
@@ -1101,7 +1108,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   const size_t smem = s->groups * group_bytes(s);
   const int threads = 32 * s->B * s->groups;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
-                                     rollout_blocks_per_sm(s->variant, s->general, threads, smem));
+                                     [&] { return rollout_blocks_per_sm(s->variant, s->general, threads, smem); });
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                  as_stream(stream), fr);
@@ -1370,7 +1377,7 @@ extern "C" int brax_batch_rollout(const brax_batch* b, int32_t T, int32_t K, con
   int device = 0;
   cudaGetDevice(&device);
   const SchedPlan pl = plan_schedule(b->sched_mode, b->sched_chunk, device, grid, T,
-                                     rollout_blocks_per_sm(variant, general, threads, smem));
+                                     [&] { return rollout_blocks_per_sm(variant, general, threads, smem); });
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, b->sched, 0, 2000000000LL, grid, L, &launch_grid, as_stream(stream));
   if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, as_stream(stream));
@@ -1517,7 +1524,7 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
   const size_t smem = backward_smem_bytes(s->B, s->P, 1);
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
-                                     backward_blocks_per_sm(variant, s->general, s->iso, threads, smem),
+                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, threads, smem); },
                                      (16 + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, fr);
@@ -1640,7 +1647,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   int device = 0;
   cudaGetDevice(&device);
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
-                                     backward_blocks_per_sm(variant, pl.general, pl.iso, pl.threads, pl.smem),
+                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, pl.threads, pl.smem); },
                                      (16 + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st);

@@ -593,14 +593,14 @@ __global__ void default_qp_kernel(const unsigned char* blob, int64_t N, const fl
 // ------------------------------------------------------------------ launchers
 template <class KernelT>
 static cudaError_t launch_k(KernelT k, const Launch& L, int grid, int threads, size_t smem, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, threads, smem, st>>>(L);
   return cudaGetLastError();
 }
 template <class KernelT>
 static int occupancy_k(KernelT k, int threads, size_t smem) {
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
   return n;

@@ -7,6 +7,14 @@
 
 namespace brax {
 
+// Let kernel k use smem bytes of dynamic shared memory: asked for only above
+// what every kernel may use (48 KB with its static part).
+template <class KernelT>
+inline cudaError_t allow_smem(KernelT k, size_t smem) {
+  if (smem <= 40 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 // Launch-bounds variants (max threads per block, min blocks per SM):
 // 0 = (384, 2), 1 = (576, 1), 2 = (1024, 1), 3 = (288, 3); the autotuner
 // (brax_tune.cu) picks one per system.

@@ -668,7 +668,7 @@ static size_t limb_smem_bytes(const LimbLaunch& l) {
 int limb_blocks_per_sm(const LimbLaunch& l) {
   const LimbKernel k = limb_kernel(l);
   const size_t smem = limb_smem_bytes(l);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 32 * l.warps, smem) != cudaSuccess) return 0;
   return n;
@@ -676,7 +676,7 @@ int limb_blocks_per_sm(const LimbLaunch& l) {
 cudaError_t launch_rollout_limb(const Launch& L, const LimbLaunch& l, int grid, cudaStream_t st) {
   const LimbKernel k = limb_kernel(l);
   const size_t smem = limb_smem_bytes(l);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, 32 * l.warps, smem, st>>>(L);
   return cudaGetLastError();

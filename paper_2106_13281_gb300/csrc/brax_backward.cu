@@ -109,7 +109,7 @@ template <bool kGeneral, bool kIso = false>
 __device__ __forceinline__ void fwd_substep(const SysP& S, const BodyP* bodies, const PairP* pairs,
                                             const PlaneP* planes, const BodyP& bp, const HingeRegs& hr,
                                             const PointRegs* pr, int b, int B, int lane, GroupMem& gm, int bar,
-                                            int nthr, Body& s, const float* act) {
+                                            int nthr, int par, Body& s, const float* act) {
   kinematic(bp, S.h, s);
   const Frame f = make_frame(bp, s);
   if (bp.flags & kPublish) {
@@ -127,13 +127,13 @@ __device__ __forceinline__ void fwd_substep(const SysP& S, const BodyP* bodies, 
   const int np = bp.n_points;
   if (kGeneral) {
     for (int i = 0; i < np; ++i) plane_point(S, bp, bp.pt[i], planes[bp.pt[i].plane], s, f, acc);
-    for (int k = b; k < S.P; k += B) pair_forward(S, bodies, pairs[k], gm, k, lane);
+    if (S.P > 0) pairs_forward(S, bodies, pairs, b, gm, par, lane);
   } else {
     plane_points_regs(S, bp, pr, planes, np < 2 ? np : 2, s, f, acc);
     for (int i = 2; !kIso && i < np; ++i) plane_point(S, bp, bp.pt[i], planes[bp.pt[i].plane], s, f, acc);
   }
   group_sync(bar, nthr);
-  integrate<kGeneral>(S, bp, gm, lane, s, f, wr, acc);
+  integrate<kGeneral>(S, bp, b, gm, par, lane, s, f, wr, acc);
 }
 
 // Reverse of one substep.  s_in: the substep's input state; g: adjoint of
@@ -142,7 +142,7 @@ template <bool kGeneral>
 __device__ __forceinline__ void bwd_substep(const SysP& S, const BodyP* bodies, const PairP* pairs,
                                             const PlaneP* planes, const BodyP& bp, const HingeRegs& hr,
                                             const PointRegs* pr, int b, int B, int lane, GroupMem& gm, BwdMem& bm,
-                                            int bar, int nthr, const Body& s_in, GBody& g, const float* act,
+                                            int bar, int nthr, int par, const Body& s_in, GBody& g, const float* act,
                                             float* gact) {
   const float h = S.h;
   // ---- forward recompute: phase K
@@ -166,7 +166,7 @@ __device__ __forceinline__ void bwd_substep(const SysP& S, const BodyP* bodies, 
   const int np = bp.n_points;
   if (kGeneral) {
     for (int i = 0; i < np; ++i) plane_point(S, bp, bp.pt[i], planes[bp.pt[i].plane], s, f, acc);
-    for (int k = b; k < S.P; k += B) pair_forward(S, bodies, pairs[k], gm, k, lane);
+    if (S.P > 0) pairs_forward(S, bodies, pairs, b, gm, par, lane);
   } else {
     plane_points_regs(S, bp, pr, planes, np < 2 ? np : 2, s, f, acc);
     for (int i = 2; i < np; ++i) plane_point(S, bp, bp.pt[i], planes[bp.pt[i].plane], s, f, acc);
@@ -175,8 +175,7 @@ __device__ __forceinline__ void bwd_substep(const SysP& S, const BodyP* bodies, 
   // ---- forward values of phase P
   int n_pair = 0;
   if (kGeneral)
-    for (int i = 0; i < bp.n_bpairs; ++i)
-      if (gm.slot4(bp.bpair[i] >> 1, 1)[lane].z != 0.f) ++n_pair;
+    if (S.P > 0) n_pair = __popc(*gm.hit(par, b, lane));
   V3 Ft = wr.F, Tt = wr.tau;
   {
     Wrench sum{Ft, Tt};
@@ -285,7 +284,7 @@ __device__ __forceinline__ void bwd_substep(const SysP& S, const BodyP* bodies, 
   if (kGeneral) {
     for (int k = b; k < S.P; k += B) {
       const PairP& prk = pairs[k];
-      if (gm.slot4(k, 1)[lane].z == 0.f) continue;
+      if (!((*gm.hit(par, prk.ba, lane) >> ((prk.geo >> 8) & 31)) & 1u)) continue;
       GSide GA, GB;
       zero(GA);
       zero(GB);
@@ -320,9 +319,9 @@ __device__ __forceinline__ void bwd_substep(const SysP& S, const BodyP* bodies, 
     gvm = gvm + mk3(o[12 * 32], o[13 * 32], o[14 * 32]);
     gwm = gwm + mk3(o[15 * 32], o[16 * 32], o[17 * 32]);
   }
-  for (int i = 0; kGeneral && i < bp.n_bpairs; ++i) {  // the own pairs' adjoints, in the body's pair order
-    const int code = bp.bpair[i];
-    if (gm.slot4(code >> 1, 1)[lane].z == 0.f) continue;  // no contact: the pair wrote nothing for this lane
+  // the adjoints of the own pairs in contact, in the body's pair order
+  for (uint32_t m = kGeneral && S.P > 0 ? *gm.hit(par, b, lane) : 0u; m; m &= m - 1) {
+    const int code = bp.bpair[__ffs(m) - 1];
     const float* o = bm.pairg + ((int64_t)code * 18) * 32 + lane;
     gx1 = gx1 + mk3(o[0], o[32], o[64]);
 #pragma unroll
@@ -464,7 +463,7 @@ __device__ __forceinline__ void bwd_substep_iso(const SysP& S, const PlaneP* pla
 // schedule (Sched; chunk_steps counts segments, chunk 0 holds the last
 // ones), one chunk of the unit of the item it takes; the state adjoint then
 // passes from chunk to chunk through the workspace.
-template <bool kGeneral, bool kIso>
+template <bool kGeneral, bool kIso, bool kShared>
 __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -494,6 +493,11 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   const Seg& sg = L.seg[si];
   const unsigned char* blob = c_pool + sg.pool_off;
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
+  if constexpr (kShared) {  // as in the forward kernel
+    blob = smem + sg.groups * bwd_group_floats(sg.B, sg.P) * sizeof(float) - sizeof(SysP);
+    copy_params(sg.blob, smem + sg.groups * bwd_group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P, S.n_planes);
+    group_sync(0, blockDim.x);
+  }
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
   const PairP* pairs = reinterpret_cast<const PairP*>(blob + blob_pairs_off(sg.B));
   const PlaneP* planes = reinterpret_cast<const PlaneP*>(blob + blob_planes_off(sg.B, sg.P));
@@ -510,12 +514,14 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   GroupMem gm = group_mem(gbase, B, 0);
   const int K = L.K, T = L.T, nsub = S.substeps;
   float* ws = sg.ws + group * ws_group_floats(B, P, K, nsub);
-  if (kGeneral) gm.slot = reinterpret_cast<float4*>(ws + (int64_t)(K + nsub) * 13 * B * 32);  // pair impulses live in the workspace
+  if (kGeneral) gm.slot = reinterpret_cast<float2*>(ws + (int64_t)(K + nsub) * 13 * B * 32);  // pair impulses live in the workspace
   BwdMem bm;
   bm.gwr = gbase + bwd_fwd_floats(B, P, false);
   bm.gpub = bm.gwr + B * 6 * 32;
   bm.gacc = bm.gpub + B * 18 * 32;
   bm.pairg = ws + ws_pairg_off(B, P, K, nsub);
+  int par = 0;  // which buffer of hit bits the substep uses; both start clear
+  if (kGeneral) *gm.hit(0, b, lane) = *gm.hit(1, b, lane) = 0u;
   const int bar = 1 + g, nthr = 32 * B;
   const BodyP& bp = bodies[b];
   const int stride = B * 32;
@@ -585,7 +591,7 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
       if (t + 1 < t1) {
         load_act(t);
         for (int k = 0; k < nsub; ++k)
-          fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, s, act);
+          fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, par ^= 1, s, act);
       }
     }
     for (int t = t1 - 1; t >= t0; --t) {
@@ -596,7 +602,7 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
       for (int k = 0; k < nsub; ++k) {
         store_body_ws(ws_subs + (int64_t)k * 13 * stride, stride, s);
         if (k + 1 < nsub)
-          fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, s, act);
+          fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, par ^= 1, s, act);
       }
       if (sg.g_torso && b == 0 && valid) {
         const float* gt = sg.g_torso + ((int64_t)t * N + env) * 3;
@@ -609,8 +615,8 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
         if (kIso)
           bwd_substep_iso(S, planes, bp, hr, pr, b, lane, gm, bm, bar, nthr, sin, gs, act, gact);
         else
-          bwd_substep<kGeneral>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bm, bar, nthr, sin, gs, act,
-                                gact);
+          bwd_substep<kGeneral>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bm, bar, nthr, par ^= 1, sin, gs,
+                                act, gact);
         __syncwarp();
         discard_state_ws(ws_subs - lane + (int64_t)k * 13 * stride, stride, lane);
       }
@@ -656,33 +662,33 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
 // groups per SM), which holds more of the adjoint's live values than the
 // 96 registers (576, 1) gives.  Each is compiled for three kinds of system:
 // hinge-only, hinge-only with isotropic inertia (bwd_substep_iso), general.
-template <int MAXT, int MINB, bool kGeneral, bool kIso>
+template <int MAXT, int MINB, bool kGeneral, bool kIso, bool kShared>
 __global__ void __launch_bounds__(MAXT, MINB) rollout_bwd_kernel(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso>(L);
+  rollout_bwd_body<kGeneral, kIso, kShared>(L);
 }
-template <bool kGeneral, bool kIso>
+template <bool kGeneral, bool kIso, bool kShared>
 __global__ void __maxnreg__(112) rollout_bwd_kernel_r112(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso>(L);
+  rollout_bwd_body<kGeneral, kIso, kShared>(L);
 }
 
 using BwdKernel = void (*)(const Launch);
-template <bool G, bool I>
+template <bool G, bool I, bool Sh>
 static BwdKernel bwd_kernel_t(int variant) {
   switch (variant) {
-    case 0: return rollout_bwd_kernel<384, 2, G, I>;
-    case 1: return rollout_bwd_kernel<576, 1, G, I>;
-    case 3: return rollout_bwd_kernel<288, 3, G, I>;
-    case 4: return rollout_bwd_kernel_r112<G, I>;
-    default: return rollout_bwd_kernel<1024, 1, G, I>;
+    case 0: return rollout_bwd_kernel<384, 2, G, I, Sh>;
+    case 1: return rollout_bwd_kernel<576, 1, G, I, Sh>;
+    case 3: return rollout_bwd_kernel<288, 3, G, I, Sh>;
+    case 4: return rollout_bwd_kernel_r112<G, I, Sh>;
+    default: return rollout_bwd_kernel<1024, 1, G, I, Sh>;
   }
 }
-static BwdKernel bwd_kernel(int variant, bool general, bool iso) {
-  if (general) return bwd_kernel_t<true, false>(variant);
-  return iso ? bwd_kernel_t<false, true>(variant) : bwd_kernel_t<false, false>(variant);
+static BwdKernel bwd_kernel(int variant, bool general, bool iso, bool shared) {
+  if (general) return shared ? bwd_kernel_t<true, false, true>(variant) : bwd_kernel_t<true, false, false>(variant);
+  return iso ? bwd_kernel_t<false, true, false>(variant) : bwd_kernel_t<false, false, false>(variant);
 }
 
-int backward_blocks_per_sm(int variant, bool general, bool iso, int threads, size_t smem) {
-  const BwdKernel k = bwd_kernel(variant, general, iso);
+int backward_blocks_per_sm(int variant, bool general, bool iso, bool shared, int threads, size_t smem) {
+  const BwdKernel k = bwd_kernel(variant, general, iso, shared);
   if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
@@ -695,8 +701,8 @@ int backward_variant_max_threads(int variant) {
 }
 
 cudaError_t launch_rollout_backward(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,
-                                    bool iso, cudaStream_t st) {
-  const BwdKernel k = bwd_kernel(variant, general, iso);
+                                    bool iso, bool shared, cudaStream_t st) {
+  const BwdKernel k = bwd_kernel(variant, general, iso, shared);
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, threads, smem, st>>>(L);

@@ -84,8 +84,8 @@ void find_limbs(SysP& S, const std::vector<BodyP>& bodies, const std::vector<Pla
   for (int l = 0; l < L; ++l) {
     const int u = r.children[l];
     if (bodies[u].n_children != 1) return;
-    S.limb_upper[l] = u;
-    S.limb_lower[l] = bodies[u].children[0];
+    S.limb_upper[l] = (uint8_t)u;
+    S.limb_lower[l] = (uint8_t)bodies[u].children[0];
   }
   auto alike = [&](const BodyP& a, const BodyP& b) {
     bool ok = a.inv_mass == b.inv_mass && a.flags == b.flags && a.k == b.k && a.c == b.c && a.ka == b.ka &&
@@ -425,6 +425,7 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
         else if (body_pcol[bi] != ci) body_multi[bi] = 1;
         BodyP& bp = bodies[side == 0 ? ba : bb];
         REQUIRE(bp.n_bpairs < BRAX_MAX_BODY_PAIRS, "body: more than BRAX_MAX_BODY_PAIRS body-body pairs");
+        pairs[idx].geo |= bp.n_bpairs << (side == 0 ? 8 : 16);
         bp.bpair[bp.n_bpairs++] = (idx << 1) | side;
         bp.flags |= kPublish | kInPair;
       }
@@ -458,7 +459,6 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
     }
   }
   for (int k = 0; k < Pb; ++k) {
-    pairs[k].geo = 0;
     if (bodies[pairs[k].ba].gtype >= 0) pairs[k].geo |= 1;
     if (bodies[pairs[k].bb].gtype >= 0) pairs[k].geo |= 2;
   }
@@ -565,6 +565,21 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
 }  // namespace
 
 namespace {
+
+// Bytes of a system's parameters when a general kernel keeps them in shared memory.
+size_t param_smem(const brax_system* s) { return (size_t)params_bytes(s->B, s->P, s->n_planes); }
+// Whether a general launch of `with` bytes of shared memory (groups and
+// parameters) fits a block.  The parameters then come from shared memory: the
+// biped's substep takes 6.7 us there and 10.8 from the constant cache (4,864
+// environments, one group an SM).
+bool fits_block(size_t with, int device) {
+  int optin = 0;
+  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return with + 64 <= (size_t)optin;
+}
 
 size_t group_bytes(const brax_system* s) { return (size_t)group_floats(s->B, s->P) * sizeof(float); }
 
@@ -987,6 +1002,18 @@ void apply_env(const brax_system* s, Seg& sg, const EnvOut* env) {
   sg.max_z = env->p->max_z;
 }
 
+// The kernel of a system in the limb layout (0: it has none): the split kernel
+// while its warps (a quarter of the wide kernel's environments each) are at
+// most 23 an SM, 14,000 quadrupeds: there it takes 25 us a step and the wide
+// kernel 25.6; beyond, the wide kernel's warps fill the SMs (measured table at
+// rollout_limb_split_kernel).
+int limb_kind(const brax_system* s, int64_t n_envs, int n_sm) {
+  if (s->n_limbs == 0 || s->pair_variant < kLimbVariant) return 0;
+  if (s->pair_variant != kLimbVariant) return s->pair_variant;
+  const int64_t per_warp = limb_warp_envs(s->n_limbs, true), split_warps = (n_envs + per_warp - 1) / per_warp;
+  return split_warps <= 23LL * n_sm ? kLimbSplit : kLimbWide;
+}
+
 int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, const float* state0,
                  const float* actions, float* state_T, float* checkpoints, float* torso_traj, int32_t* contact_count,
                  void* stream, const EnvOut* env, const FixedRegion& fr = FixedRegion{}) {
@@ -1005,22 +1032,18 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   // is switched on, checkpointing rollouts included: the reverse pass
   // rebuilds a checkpoint segment's step states with the kernel that wrote
   // the checkpoints (rollout_backward_impl), so gradients do not depend on K.
-  if (s->pair_mode == 1 && s->pair_variant >= kLimbVariant) {
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess) {
-      cudaGetLastError();
-      n_sm = 1;
-    }
+  int n_sm = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess) {
+    cudaGetLastError();
+    n_sm = 1;
+  }
+  const int kind = s->pair_mode == 1 ? limb_kind(s, n_envs, n_sm) : 0;
+  if (kind != 0) {
     LimbLaunch ll;
     ll.n_limbs = s->n_limbs;
     ll.frozen = s->frozen;
     ll.env = env != nullptr;
-    // The split kernel while its warps (a quarter of the wide kernel's
-    // environments each) are at most 23 an SM, 14,000 quadrupeds: there it
-    // takes 25 us a step and the wide kernel 25.6; beyond, the wide kernel's
-    // warps fill the SMs (measured table at rollout_limb_split_kernel).
-    const int64_t split_warps = (n_envs + limb_warp_envs(s->n_limbs, true) - 1) / limb_warp_envs(s->n_limbs, true);
-    ll.split = s->pair_variant == kLimbVariant ? split_warps <= 23LL * n_sm : s->pair_variant == kLimbSplit;
+    ll.split = kind == kLimbSplit;
     // blocks of one warp until every SM has one, then up to four (one per
     // scheduler of an SM)
     const int64_t per_warp = limb_warp_envs(s->n_limbs, ll.split), n_warps = (n_envs + per_warp - 1) / per_warp;
@@ -1050,8 +1073,11 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout");
   }
   if (s->pair_mode == 1) {
-    Seg sg = make_seg(s, s->pair_groups, n_envs);
-    const int64_t per_cta = 64LL * s->pair_groups;
+    // (the limb layout's rule found the body layout faster: its default launch)
+    const bool picked = s->pair_variant >= kLimbVariant;
+    const int groups = picked ? 1 : s->pair_groups, pvariant = picked ? 0 : s->pair_variant;
+    Seg sg = make_seg(s, groups, n_envs);
+    const int64_t per_cta = 64LL * groups;
     const int64_t grid = (n_envs + per_cta - 1) / per_cta;
     if (grid > 0x7fffffff) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout: too many environments");
     sg.cta_begin = 0;
@@ -1064,9 +1090,9 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     sg.ccount = contact_count;
     apply_env(s, sg, env);
     L.seg[0] = sg;
-    size_t smem = s->pair_groups * pair_group_bytes(s->B, s->A);
+    size_t smem = groups * pair_group_bytes(s->B, s->A);
     if (checkpoints) {  // checkpoint staging buffers, [64][B][13] floats a group, when they fit
-      const size_t with = smem + (size_t)s->pair_groups * 64 * s->B * 13 * sizeof(float);
+      const size_t with = smem + (size_t)groups * 64 * s->B * 13 * sizeof(float);
       int optin = 0;
       if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device) != cudaSuccess) {
         cudaGetLastError();
@@ -1077,9 +1103,9 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
         L.seg[0].ck_stage = 1;
       }
     }
-    const int threads = 32 * s->B * s->pair_groups;
+    const int threads = 32 * s->B * groups;
     const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
-                                       [&] { return pair_blocks_per_sm(s->pair_variant, threads, smem); });
+                                       [&] { return pair_blocks_per_sm(pvariant, threads, smem); });
     int64_t launch_grid;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                    as_stream(stream), fr);
@@ -1087,7 +1113,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     s->last_chunks = L.sc.n_chunks;
     s->last_chunk_steps = L.sc.chunk_steps;
     if (e == cudaSuccess)
-      e = launch_rollout_pair(L, (int)launch_grid, threads, smem, s->pair_variant,
+      e = launch_rollout_pair(L, (int)launch_grid, threads, smem, pvariant,
                               reinterpret_cast<const SysP*>(s->blob.data())->flat != 0, as_stream(stream));
     return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout");
   }
@@ -1105,17 +1131,19 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   sg.ccount = contact_count;
   apply_env(s, sg, env);
   L.seg[0] = sg;
-  const size_t smem = s->groups * group_bytes(s);
+  size_t smem = s->groups * group_bytes(s);
+  const bool shared = s->general && fits_block(smem + param_smem(s), s->device);
+  if (shared) smem += param_smem(s);
   const int threads = 32 * s->B * s->groups;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
-                                     [&] { return rollout_blocks_per_sm(s->variant, s->general, threads, smem); });
+                                     [&] { return rollout_blocks_per_sm(s->variant, s->general, shared, threads, smem); });
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                  as_stream(stream), fr);
   s->last_grid = launch_grid;
   s->last_chunks = L.sc.n_chunks;
   s->last_chunk_steps = L.sc.chunk_steps;
-  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, s->variant, s->general, as_stream(stream));
+  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, s->variant, s->general, shared, as_stream(stream));
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout");
 }
 
@@ -1259,6 +1287,16 @@ int brax_sync_status(const brax_system* s, void* stream) {
 namespace {
 // Groups per block for system s when a block has `warps` warps.
 int batch_groups(const brax_system* s, int warps) { return std::max(1, std::min(15, warps / s->B)); }
+int64_t batch_blocks(const brax_system* s, int warps, int64_t n_envs) {
+  const int64_t per = 32LL * batch_groups(s, warps);
+  return (n_envs + per - 1) / per;
+}
+// The systems in the order their blocks start.
+std::vector<int> batch_order(const brax_batch* b) {
+  std::vector<int> order(b->sys.size());
+  for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+  return order;
+}
 }  // namespace
 
 extern "C" {
@@ -1324,30 +1362,33 @@ int brax_batch_offsets(const brax_batch* b, int32_t T, int32_t K, int32_t i, int
 namespace brax_batch_impl {
 // Fill a launch table for the batch; pointers offset per system.
 int make_launch(const brax_batch* b, int32_t T, int32_t K, Launch& L, int* grid, int* threads, size_t* smem,
-                bool* general) {
+                size_t* smem_with, bool* general) {
   *general = false;
   std::memset(&L, 0, sizeof(L));
   L.n_segs = (int)b->sys.size();
   L.T = T;
   L.K = K;
   int cta = 0;
-  size_t sm = 0;
-  for (int i = 0; i < L.n_segs; ++i) {
+  size_t sm = 0, sw = 0;  // shared memory without and with the parameters
+  const std::vector<int> order = batch_order(b);
+  for (int j = 0; j < L.n_segs; ++j) {
+    const int i = order[j];
     const brax_system* s = b->sys[i];
     const int G = batch_groups(s, b->warps);
     Seg sg = make_seg(s, G, b->n_envs[i]);
-    const int64_t per = 32LL * G;
-    const int64_t nb = (b->n_envs[i] + per - 1) / per;
+    const int64_t nb = batch_blocks(s, b->warps, b->n_envs[i]);
     sg.cta_begin = cta;
     sg.cta_end = cta + (int)nb;
     cta += (int)nb;
     sm = std::max(sm, (size_t)G * group_bytes(s));
+    sw = std::max(sw, (size_t)G * group_bytes(s) + param_smem(s));
     *general = *general || s->general;
-    L.seg[i] = sg;
+    L.seg[j] = sg;
   }
   *grid = cta;
   *threads = 32 * b->warps;
   *smem = sm;
+  *smem_with = sw;
   return BRAX_OK;
 }
 }  // namespace brax_batch_impl
@@ -1359,28 +1400,31 @@ extern "C" int brax_batch_rollout(const brax_batch* b, int32_t T, int32_t K, con
   if (K < 1) K = 1;
   Launch L;
   int grid, threads;
-  size_t smem;
+  size_t smem, smem_with;
   bool general;
-  brax_batch_impl::make_launch(b, T, K, L, &grid, &threads, &smem, &general);
-  for (int i = 0; i < L.n_segs; ++i) {
+  brax_batch_impl::make_launch(b, T, K, L, &grid, &threads, &smem, &smem_with, &general);
+  const std::vector<int> order = batch_order(b);
+  for (int j = 0; j < L.n_segs; ++j) {
     int64_t so, ao, to, co;
-    brax_batch_offsets(b, T, K, i, &so, &ao, &to, &co);
-    L.seg[i].state0 = state0 + so;
-    L.seg[i].actions = actions ? actions + ao : nullptr;
-    L.seg[i].state_T = state_T + so;
-    L.seg[i].ckpt = checkpoints ? checkpoints + co : nullptr;
-    L.seg[i].torso = torso_traj ? torso_traj + to : nullptr;
+    brax_batch_offsets(b, T, K, order[j], &so, &ao, &to, &co);
+    L.seg[j].state0 = state0 + so;
+    L.seg[j].actions = actions ? actions + ao : nullptr;
+    L.seg[j].state_T = state_T + so;
+    L.seg[j].ckpt = checkpoints ? checkpoints + co : nullptr;
+    L.seg[j].torso = torso_traj ? torso_traj + to : nullptr;
   }
   if (grid == 0) return BRAX_OK;
   const int variant = pick_variant(threads);
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_batch_rollout: block too large");
   int device = 0;
   cudaGetDevice(&device);
+  const bool shared = general && fits_block(smem_with, device);
+  if (shared) smem = smem_with;
   const SchedPlan pl = plan_schedule(b->sched_mode, b->sched_chunk, device, grid, T,
-                                     [&] { return rollout_blocks_per_sm(variant, general, threads, smem); });
+                                     [&] { return rollout_blocks_per_sm(variant, general, shared, threads, smem); });
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, b->sched, 0, 2000000000LL, grid, L, &launch_grid, as_stream(stream));
-  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, as_stream(stream));
+  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, shared, as_stream(stream));
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout");
 }
 
@@ -1521,15 +1565,17 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
       (s->bwd_variant >= 0 && threads <= backward_variant_max_threads(s->bwd_variant)) ? s->bwd_variant
                                                                                         : pick_bwd_variant(threads);
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout_backward: system too large for one block");
-  const size_t smem = backward_smem_bytes(s->B, s->P, 1);
+  size_t smem = backward_smem_bytes(s->B, s->P, 1);
+  const bool shared = s->general && fits_block(smem + param_smem(s), s->device);
+  if (shared) smem += param_smem(s);
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
-                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, threads, smem); },
+                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, threads, smem); },
                                      (16 + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, fr);
   if (e == cudaSuccess)
-    e = launch_rollout_backward(L, (int)launch_grid, threads, smem, variant, s->general, s->iso, st);
+    e = launch_rollout_backward(L, (int)launch_grid, threads, smem, variant, s->general, s->iso, shared, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout_backward");
 }
 }  // namespace
@@ -1561,33 +1607,32 @@ namespace {
 // groups of 32 environments, its workspace block starts at ws_off[i].
 struct BwdBatchPlan {
   int grid = 0, threads = 0;
-  size_t smem = 0, ws_bytes = 0;
+  size_t smem = 0, smem_with = 0, ws_bytes = 0;  // smem_with: with the parameters in shared memory
   bool general = false, iso = true;
-  std::vector<int> groups, cta_begin, cta_end;
+  std::vector<int> groups, blocks;  // by system
+  std::vector<int> order;           // the systems as their blocks start
   std::vector<size_t> ws_off;
 };
 BwdBatchPlan plan_batch_backward(const brax_batch* b, int32_t K) {
   BwdBatchPlan pl;
   pl.threads = 32 * b->warps;
-  int cta = 0;
+  pl.order = batch_order(b);
   for (size_t i = 0; i < b->sys.size(); ++i) {
     const brax_system* s = b->sys[i];
     const SysP* S = reinterpret_cast<const SysP*>(s->blob.data());
     const int G = batch_groups(s, b->warps);
-    const int64_t per = 32LL * G;
-    const int nb = (int)((b->n_envs[i] + per - 1) / per);
+    const int nb = (int)batch_blocks(s, b->warps, b->n_envs[i]);
     pl.groups.push_back(G);
-    pl.cta_begin.push_back(cta);
-    pl.cta_end.push_back(cta + nb);
-    cta += nb;
+    pl.blocks.push_back(nb);
+    pl.grid += nb;
     pl.ws_off.push_back(pl.ws_bytes);
     const size_t wb = (size_t)nb * G * (size_t)backward_ws_floats_per_group(s->B, s->P, K, S->substeps) * sizeof(float);
     pl.ws_bytes += (wb + 255) & ~size_t(255);
     pl.smem = std::max(pl.smem, backward_smem_bytes(s->B, s->P, G));
+    pl.smem_with = std::max(pl.smem_with, backward_smem_bytes(s->B, s->P, G) + param_smem(s));
     pl.general = pl.general || s->general;
     pl.iso = pl.iso && s->iso;
   }
-  pl.grid = cta;
   return pl;
 }
 }  // namespace
@@ -1626,12 +1671,14 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   L.n_segs = (int)b->sys.size();
   L.T = T;
   L.K = K;
-  for (int i = 0; i < L.n_segs; ++i) {
+  int cta = 0;
+  for (int j = 0; j < L.n_segs; ++j) {
+    const int i = pl.order[j];
     int64_t so, ao, to, co;
     brax_batch_offsets(b, T, K, i, &so, &ao, &to, &co);
     Seg sg = make_seg(b->sys[i], pl.groups[i], b->n_envs[i]);
-    sg.cta_begin = pl.cta_begin[i];
-    sg.cta_end = pl.cta_end[i];
+    sg.cta_begin = cta;
+    sg.cta_end = cta += pl.blocks[i];
     sg.state0 = state0 + so;
     sg.actions = actions ? actions + ao : nullptr;
     sg.ckpt = const_cast<float*>(checkpoints) + co;
@@ -1640,19 +1687,21 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
     sg.g_actions = g_actions ? g_actions + ao : nullptr;
     sg.g_state0 = g_state0 ? g_state0 + so : nullptr;
     sg.ws = reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + pl.ws_off[i]);
-    L.seg[i] = sg;
+    L.seg[j] = sg;
   }
   const int variant = pick_bwd_variant(pl.threads);
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_batch_rollout_backward: block too large");
   int device = 0;
   cudaGetDevice(&device);
+  const bool shared = pl.general && fits_block(pl.smem_with, device);
+  const size_t smem = shared ? pl.smem_with : pl.smem;
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
-                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, pl.threads, pl.smem); },
+                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.threads, smem); },
                                      (16 + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st);
   if (e == cudaSuccess)
-    e = launch_rollout_backward(L, (int)launch_grid, pl.threads, pl.smem, variant, pl.general, pl.iso, st);
+    e = launch_rollout_backward(L, (int)launch_grid, pl.threads, smem, variant, pl.general, pl.iso, shared, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout_backward");
 }
 

@@ -237,30 +237,56 @@ __device__ __forceinline__ void bar_arrive(int id, int nthreads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Copy a system's body, pair and plane parameters (what follows SysP in its
+// blob) to shared memory; the whole block takes part, and synchronises after.
+__device__ __forceinline__ void copy_params(const unsigned char* blob, unsigned char* dst, int B, int P, int n_planes) {
+  const uint4* src = reinterpret_cast<const uint4*>(blob + blob_bodies_off());
+  uint4* d = reinterpret_cast<uint4*>(dst);
+  for (int i = threadIdx.x; i < params_bytes(B, P, n_planes) / 16; i += blockDim.x) d[i] = __ldg(src + i);
+}
+
 // ------------------------------------------------------------------ group shared memory
 // Four consecutive fields of one lane form one float4, so a warp moves a
 // chunk with one 16-byte access per lane (512 contiguous bytes, no bank
 // conflict) instead of four scalar accesses.
 // pub  [B][6][32] float4: a publishing body's post-kinematic
 //                         (x, R0) (R1..R4) (R5..R8) (v, w.x) (w.y, w.z, Ii0, Ii1) (Ii2..Ii5)
-// react[B][2][32] float4: a child's joint reaction on its parent (F, tau.x) (tau.y, tau.z, -, -)
-// slot [P][2][32] float4: a body-body pair's (J, p.x) (p.y, p.z, active flag, -)
+// react[B][2][32] float4: a child's joint reaction on its parent (F, tau.x) (tau.y, tau.z, hits, hits)
+// slot [P][3][32] float2: a body-body pair's (J.x, J.y) (J.z, p.x) (p.y, p.z),
+//                         written where it is in contact; the free half of a
+//                         body's second react chunk holds its hit bits: bit i,
+//                         its i-th pair is in contact; .z and .w in turn,
+//                         substep by substep
 struct GroupMem {
   float4* pub;
   float4* react;
-  float4* slot;
+  float2* slot;
   int* cnt;
+  __device__ __forceinline__ uint32_t* hit(int par, int b, int lane) {
+    return reinterpret_cast<uint32_t*>(react4(b, 1) + lane) + 2 + par;
+  }
   __device__ __forceinline__ float4* pub4(int b, int c) { return pub + (b * (kPubFields / 4) + c) * 32; }
   __device__ __forceinline__ float4* react4(int b, int c) { return react + (b * (kReactFields / 4) + c) * 32; }
-  __device__ __forceinline__ float4* slot4(int k, int c) { return slot + (k * (kSlotFields / 4) + c) * 32; }
+  __device__ __forceinline__ void put_slot(int k, int lane, V3 J, V3 p) {
+    float2* q = slot + k * (kSlotFields / 2) * 32 + lane;
+    q[0] = make_float2(J.x, J.y);
+    q[32] = make_float2(J.z, p.x);
+    q[64] = make_float2(p.y, p.z);
+  }
+  __device__ __forceinline__ void get_slot(int k, int lane, V3& J, V3& p) const {
+    const float2* q = slot + k * (kSlotFields / 2) * 32 + lane;
+    const float2 a = q[0], b = q[32], c = q[64];
+    J = mk3(a.x, a.y, b.x);
+    p = mk3(b.y, c.x, c.y);
+  }
 };
 // base must be 16-byte aligned.
 __device__ __forceinline__ GroupMem group_mem(float* base, int B, int P) {
   GroupMem m;
   m.pub = reinterpret_cast<float4*>(base);
   m.react = m.pub + B * (kPubFields / 4) * 32;
-  m.slot = m.react + B * (kReactFields / 4) * 32;
-  m.cnt = reinterpret_cast<int*>(m.slot + P * (kSlotFields / 4) * 32);
+  m.slot = reinterpret_cast<float2*>(m.react + B * (kReactFields / 4) * 32);
+  m.cnt = reinterpret_cast<int*>(m.slot + P * (kSlotFields / 2) * 32);
   return m;
 }
 __device__ __forceinline__ float2 lo2(float4 a) { return make_float2(a.x, a.y); }

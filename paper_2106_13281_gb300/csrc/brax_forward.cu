@@ -23,7 +23,7 @@ template <bool kGeneral>
 __device__ __forceinline__ int substep_forward(const SysP& S, const BodyP* bodies, const PairP* pairs,
                                                const PlaneP* planes, const BodyP& bp, const HingeRegs& hr,
                                                const PointRegs* pr, int b, int B, int lane, GroupMem& gm, int bar,
-                                               int nthr, bool tree, Body& s, const float* act) {
+                                               int nthr, bool tree, int par, Body& s, const float* act) {
   kinematic(bp, S.h, s);
   const Frame f = make_frame(bp, s);
   if (!kGeneral && tree) {
@@ -51,7 +51,7 @@ __device__ __forceinline__ int substep_forward(const SysP& S, const BodyP* bodie
       bar_arrive(pid + 1, pn);
     }
     if (parent_of) group_sync(3 + 2 * bp.tree_slot, my_n);
-    integrate<false>(S, bp, gm, lane, s, f, wr, acc);
+    integrate<false>(S, bp, b, gm, par, lane, s, f, wr, acc);
     return counted;
   }
   if (bp.flags & kPublish) {
@@ -74,10 +74,9 @@ __device__ __forceinline__ int substep_forward(const SysP& S, const BodyP* bodie
     for (int i = 2; i < np; ++i) plane_point(S, bp, bp.pt[i], planes[bp.pt[i].plane], s, f, acc);
   }
   int counted = acc.n;
-  if (kGeneral)
-    for (int k = b; k < S.P; k += B) counted += pair_forward(S, bodies, pairs[k], gm, k, lane);
+  if (kGeneral && S.P > 0) counted += pairs_forward(S, bodies, pairs, b, gm, par, lane);
   group_sync(bar, nthr);
-  integrate<kGeneral>(S, bp, gm, lane, s, f, wr, acc);
+  integrate<kGeneral>(S, bp, b, gm, par, lane, s, f, wr, acc);
   return counted;
 }
 
@@ -87,7 +86,12 @@ __device__ __forceinline__ int substep_forward(const SysP& S, const BodyP* bodie
 // runs one unit (a block-sized set of environment groups of one segment):
 // unit blockIdx.x for the whole rollout, or, under a chunked schedule
 // (Sched), one chunk of the unit of the item it takes.
-template <int MAXT, int MINB, bool kGeneral, bool kEnv>
+//
+// kShared (general systems): the bodies', pairs' and planes' parameters are
+// read from a copy in shared memory.  A general system's warps read about 28 KB
+// of them a substep, each its own body's and pairs', far more than the constant
+// cache holds (measured on the biped: 20-29 % of its requests miss).
+template <int MAXT, int MINB, bool kGeneral, bool kEnv, bool kShared>
 __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_constant__ Launch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -119,6 +123,11 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
   const Seg& sg = L.seg[si];
   const unsigned char* blob = c_pool + sg.pool_off;
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
+  if constexpr (kShared) {
+    blob = smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float) - sizeof(SysP);
+    copy_params(sg.blob, smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P, S.n_planes);
+    group_sync(0, blockDim.x);
+  }
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
   const PairP* pairs = reinterpret_cast<const PairP*>(blob + blob_pairs_off(sg.B));
   const PlaneP* planes = reinterpret_cast<const PlaneP*>(blob + blob_planes_off(sg.B, sg.P));
@@ -136,6 +145,8 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
   // tree barriers need the block to be exactly one group (their ids are per block)
   const bool tree = !kGeneral && sg.groups == 1 && (int)blockDim.x == 32 * B && tree_barriers_fit(S.n_parents);
   if (b == 0) gm.cnt[lane] = 0;
+  int par = 0;  // which buffer of hit bits the substep uses; both start clear
+  if (kGeneral) *gm.hit(0, b, lane) = *gm.hit(1, b, lane) = 0u;
   if (sg.ccount) group_sync(bar, nthr);
 
   Body s;
@@ -171,8 +182,8 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
     }
     if (kEnv && b == 0) gm.react4(0, 0)[lane].x = s.x.x;  // the root's x before the step (its react slot is free)
     for (int k = 0; k < nsub; ++k)
-      ccount += substep_forward<kGeneral>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, tree, s,
-                                          act);
+      ccount += substep_forward<kGeneral>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, tree,
+                                          par ^= 1, s, act);
     if (sg.torso && b == 0 && valid) {
       float* tp = sg.torso + ((int64_t)t * N + env) * 3;
       tp[0] = s.x.x;
@@ -185,7 +196,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
       // leaves its final angular velocity where its children read its
       // published state (its rotation there is already the final one: only
       // velocities change after the kinematic integrator); a joint's child
-      // leaves its actions' squared clamped values beside its reaction.
+      // leaves its actions' squared clamped values where the inertia was published.
       if (bp.flags & kPublish) {
         gm.pub4(b, 3)[lane].w = s.w.x;
         st2(gm.pub4(b, 4) + lane, s.w.y, s.w.z);
@@ -198,7 +209,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
             const float u = clamp1(act[a]);
             c2 = fmaf(u, u, c2);
           }
-        gm.react4(b, 1)[lane].z = c2;
+        gm.pub4(b, 4)[lane].z = c2;
       }
       group_sync(bar, nthr);
       float* ob = sg.obs + ((int64_t)t * N + env) * sg.obs_dim;
@@ -216,7 +227,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
       if (b == 0) {
         float ctrl = 0.f;
         for (int c = 1; c < B; ++c)
-          if (bodies[c].flags & kHasParent) ctrl += gm.react4(c, 1)[lane].z;
+          if (bodies[c].flags & kHasParent) ctrl += gm.pub4(c, 4)[lane].z;
         bool done = false;
         if (valid)
           done = root_env(sg, s, gm.react4(0, 0)[lane].x, ctrl, ob, sg.reward + (int64_t)t * N + env,
@@ -611,36 +622,29 @@ static int occupancy_k(KernelT k, int threads, size_t smem) {
 // A rollout with the environment layer (Seg::obs) runs the kernels compiled
 // with it, in the (576, 1) launch, or (1024, 1) for larger blocks; the
 // others are compiled without it, so plain rollouts carry none of its code.
-template <bool G>
-static cudaError_t launch_rollout_g(const Launch& L, int grid, int threads, size_t smem, int variant, cudaStream_t st) {
-  if (L.seg[0].obs)
-    return threads <= 576 ? launch_k(rollout_kernel<576, 1, G, true>, L, grid, threads, smem, st)
-                          : launch_k(rollout_kernel<1024, 1, G, true>, L, grid, threads, smem, st);
+// shared: a general system's parameters in shared memory (smem includes them).
+using RolloutKernel = void (*)(const Launch);
+template <bool G, bool Sh>
+static RolloutKernel rollout_kernel_t(int variant, int threads, bool env) {
+  if (env) return threads <= 576 ? rollout_kernel<576, 1, G, true, Sh> : rollout_kernel<1024, 1, G, true, Sh>;
   switch (variant) {
-    case 0: return launch_k(rollout_kernel<384, 2, G, false>, L, grid, threads, smem, st);
-    case 1: return launch_k(rollout_kernel<576, 1, G, false>, L, grid, threads, smem, st);
-    case 3: return launch_k(rollout_kernel<288, 3, G, false>, L, grid, threads, smem, st);
-    default: return launch_k(rollout_kernel<1024, 1, G, false>, L, grid, threads, smem, st);
+    case 0: return rollout_kernel<384, 2, G, false, Sh>;
+    case 1: return rollout_kernel<576, 1, G, false, Sh>;
+    case 3: return rollout_kernel<288, 3, G, false, Sh>;
+    default: return rollout_kernel<1024, 1, G, false, Sh>;
   }
 }
-cudaError_t launch_rollout(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,
+static RolloutKernel rollout_kernel_of(int variant, bool general, bool shared, int threads, bool env) {
+  if (!general) return rollout_kernel_t<false, false>(variant, threads, env);
+  return shared ? rollout_kernel_t<true, true>(variant, threads, env) : rollout_kernel_t<true, false>(variant, threads, env);
+}
+cudaError_t launch_rollout(const Launch& L, int grid, int threads, size_t smem, int variant, bool general, bool shared,
                            cudaStream_t st) {
-  return general ? launch_rollout_g<true>(L, grid, threads, smem, variant, st)
-                 : launch_rollout_g<false>(L, grid, threads, smem, variant, st);
+  return launch_k(rollout_kernel_of(variant, general, shared, threads, L.seg[0].obs != nullptr), L, grid, threads, smem,
+                  st);
 }
-
-template <bool G>
-static int rollout_blocks_per_sm_g(int variant, int threads, size_t smem) {
-  switch (variant) {
-    case 0: return occupancy_k(rollout_kernel<384, 2, G, false>, threads, smem);
-    case 1: return occupancy_k(rollout_kernel<576, 1, G, false>, threads, smem);
-    case 3: return occupancy_k(rollout_kernel<288, 3, G, false>, threads, smem);
-    default: return occupancy_k(rollout_kernel<1024, 1, G, false>, threads, smem);
-  }
-}
-int rollout_blocks_per_sm(int variant, bool general, int threads, size_t smem) {
-  return general ? rollout_blocks_per_sm_g<true>(variant, threads, smem)
-                 : rollout_blocks_per_sm_g<false>(variant, threads, smem);
+int rollout_blocks_per_sm(int variant, bool general, bool shared, int threads, size_t smem) {
+  return occupancy_k(rollout_kernel_of(variant, general, shared, threads, false), threads, smem);
 }
 
 // Two-environments-per-thread variants: 0: (288, 2)  1: (576, 1)  2: (1024, 1)  3: (288, 3)

@@ -35,7 +35,8 @@ struct PointP {
   int32_t pad;
 };
 
-struct BodyP {
+// (16-byte aligned, so that neighbouring fields load together from shared memory)
+struct alignas(16) BodyP {
   float inv_mass;
   float inv_I[3];
   uint32_t flags;
@@ -60,7 +61,7 @@ struct BodyP {
   int32_t n_points;
   PointP pt[BRAX_MAX_POINTS];
   int32_t n_bpairs;
-  int32_t bpair[BRAX_MAX_BODY_PAIRS];  // (pair index << 1) | side; side 0: +J (body a), 1: -J (body b)
+  int32_t bpair[BRAX_MAX_BODY_PAIRS];  // (pair index << 1) | side; side 0: +J (body a), 1: -J (body b); ascending
   // default_qp: rest pose for roots
   float rest_pos[3];
   float rest_rot[4];
@@ -70,7 +71,8 @@ struct BodyP {
   // The body's collider in body-body pairs when it has exactly one (-1: none
   // or several): its world geometry is computed once per substep and
   // published (capsule: g0, g1 = segment end points; box: g0 = centre,
-  // g1 = axes, row-major), instead of once per pair.
+  // g1 = axes, row-major), instead of once per pair; with the centre of its
+  // bounding sphere.
   int32_t gtype;  // -1, 0 capsule, 1 box
   float g0[3];
   float g1[9];
@@ -81,10 +83,11 @@ enum PairType : int32_t { kCapsuleCapsule = 0, kCapsuleBox = 1 };
 // A body-body pair: capsule a (segment a0..a1 in body a's frame, radius ra)
 // against capsule b (segment b0..b1, radius rb) or against box b (centre b0,
 // half extents b1, axes bR columns, all in body b's frame).
-struct PairP {
+struct alignas(16) PairP {
   int32_t type;
   int32_t ba, bb;
-  int32_t geo;  // bit 0 / bit 1: body a's / body b's collider geometry is published by the body
+  int32_t geo;  // bit 0 / bit 1: body a's / body b's collider geometry is published by the body;
+                // bits 8..12 / 16..20: the pair's place in body a's / body b's bpair
   float mu, e;
   float ra, rb;
   float a0[3], a1[3];
@@ -105,7 +108,7 @@ struct PlaneP {
   float n[3];
 };
 
-struct SysP {
+struct alignas(16) SysP {
   int32_t B, J, A, D, P, n_planes, substeps, average;
   float h, beta_h, eps;  // beta_h = baumgarte / h
   float lin_damp;        // global linear damping (1/s) of the potential integrator, 0: none
@@ -124,7 +127,7 @@ struct SysP {
   // Limb layout (brax_limb.cuh): n_limbs > 0 when the system is one root with
   // n_limbs limbs of two hinged bodies each, alike up to their geometry.
   int32_t n_limbs, limb_root;
-  int32_t limb_upper[BRAX_MAX_CHILDREN], limb_lower[BRAX_MAX_CHILDREN];  // in the order of the root's children
+  uint8_t limb_upper[BRAX_MAX_CHILDREN], limb_lower[BRAX_MAX_CHILDREN];  // in the order of the root's children
 };
 
 // Two environments per thread (systems with hinge joints only and at most
@@ -161,13 +164,17 @@ __host__ __device__ inline int blob_bytes(int B, int P, int n_planes) {
   int b = blob_planes_off(B, P) + n_planes * (int)sizeof(PlaneP);
   return (b + 15) & ~15;
 }
+// Of it, what follows SysP: the bodies, pairs and planes.
+__host__ __device__ inline int params_bytes(int B, int P, int n_planes) {
+  return blob_bytes(B, P, n_planes) - blob_bodies_off();
+}
 // The paired section (SysP2, BodyP2[B]) starts at blob_bytes(B, P, n_planes).
 __host__ __device__ inline int blob_pair_bytes(int B) { return (int)sizeof(SysP2) + B * (int)sizeof(BodyP2); }
 
 // Shared memory of one group of 32 environments (floats), after the blob.
 constexpr int kPubFields = 36;    // x[3], R[9], v[3], w[3], Ii[6], pair geometry[12]: nine float4 per lane
-constexpr int kReactFields = 8;   // F[3], tau[3], 2 pad: two float4 per lane
-constexpr int kSlotFields = 8;    // J[3], p[3], active flag, pad: two float4 per lane
+constexpr int kReactFields = 8;   // F[3], tau[3], two words of hit bits (GroupMem::hit): two float4 per lane
+constexpr int kSlotFields = 6;    // J[3], p[3]: three float2 per lane
 // Tree barriers (one group per block): parent slot k owns named barrier
 // 2 + 2k (its published state, parent -> children) and 3 + 2k (its
 // children's reactions, children -> parent); each counts the parent's warp and

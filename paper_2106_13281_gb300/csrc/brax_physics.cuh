@@ -139,8 +139,10 @@ __device__ __forceinline__ void publish(GroupMem& gm, int b, int lane, const Bod
     if (bp.gtype == 0) {
       V3 P, d;
       capsule_world(f.R, s.x, bp.g0, bp.g1, P, d);
+      const V3 m = fma3(0.5f, d, P);  // the bounding sphere's centre (a box has its own centre in the first chunk)
       p[192] = make_float4(P.x, P.y, P.z, d.x);
       st2(p + 224, d.y, d.z);
+      p[256] = make_float4(m.x, m.y, m.z, 0.f);
     } else if (bp.gtype == 1) {
       M3 Rb;
       V3 cb;
@@ -542,9 +544,16 @@ __device__ __forceinline__ float seg_box_param(V3 Pl, V3 dl, const float* he) {
   return fmaf(tr - tl, __fdividef(gl, gl - gr), tl);
 }
 
-// Detect one body-body pair; on contact compute the impulse on body a and
-// write (J, p, 1) to the pair's slot, else (0, 0, 0).
-__device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, const PairP& pr, GroupMem& gm,
+// Whether a pair's bounding spheres are disjoint in every environment of the
+// warp (broadphase of a pair whose bodies do not publish their geometry).
+__device__ __forceinline__ bool apart(V3 a, V3 b, float bound2) {
+  const V3 d = a - b;
+  return __all_sync(0xffffffffu, dot(d, d) > bound2);
+}
+
+// Detect one body-body pair; on contact compute the impulse on body a, write
+// (J, p) to the pair's slot and set both bodies' hit bits.
+__device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, const PairP& pr, GroupMem& gm, int par,
                                             int k, int lane) {
   // detection needs only the colliders' world geometry: published by the
   // bodies (computed once per substep), else computed here
@@ -566,16 +575,7 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
       const Pub Bq = read_pub(gm, pr.bb, lane);
       capsule_world(Bq.R, Bq.x, pr.b0, pr.b1, P2, d2);
     }
-    // broadphase (Sec. 7.2's future work): disjoint bounding spheres cannot
-    // touch; when no environment of the warp needs the narrow phase, skip it
-    // (an environment that does not need it would find no contact there)
-    const V3 dm = fma3(0.5f, d1, P1) - fma3(0.5f, d2, P2);
-    if (__all_sync(0xffffffffu, dot(dm, dm) > pr.bound2)) {
-      float4* sl = gm.slot4(k, 0) + lane;
-      sl[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-      sl[32] = make_float4(0.f, 0.f, 0.f, 0.f);
-      return 0;
-    }
+    if ((pr.geo & 3) != 3 && apart(fma3(0.5f, d1, P1), fma3(0.5f, d2, P2), pr.bound2)) return 0;
     float sp, tp;
     segment_closest(P1, d1, P2, d2, sp, tp);
     const V3 c1 = fma3(sp, d1, P1), c2 = fma3(tp, d2, P2);
@@ -599,13 +599,7 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
       const Pub Bq = read_pub(gm, pr.bb, lane);
       box_world(Bq.R, Bq.x, pr.b0, pr.bR, Rb, cb);
     }
-    const V3 dm = fma3(0.5f, d1, P1) - cb;  // broadphase, as for two capsules
-    if (__all_sync(0xffffffffu, dot(dm, dm) > pr.bound2)) {
-      float4* sl = gm.slot4(k, 0) + lane;
-      sl[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-      sl[32] = make_float4(0.f, 0.f, 0.f, 0.f);
-      return 0;
-    }
+    if ((pr.geo & 3) != 3 && apart(fma3(0.5f, d1, P1), cb, pr.bound2)) return 0;
     const V3 Pl = mulT(Rb, P1 - cb);
     const V3 dl = mulT(Rb, d1);
     const float* he = pr.b1;
@@ -642,12 +636,7 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
       hit = true;
     }
   }
-  float4* sl = gm.slot4(k, 0) + lane;
-  if (!hit) {
-    sl[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    sl[32] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return 0;
-  }
+  if (!hit) return 0;
   const Pub A = read_pub(gm, pr.ba, lane);
   const Pub Bq = read_pub(gm, pr.bb, lane);
   const BodyP& ba = bodies[pr.ba];
@@ -657,11 +646,7 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
   const V3 la = p - A.x, lb = p - Bq.x;
   const V3 u = (A.v + cross(A.w, la)) - (Bq.v + cross(Bq.w, lb));
   const float kn = eff_mass(ba.flags, ba.inv_mass, Ia, la, n) + eff_mass(bb.flags, bb.inv_mass, Ib, lb, n);
-  if (!(kn > 0.f)) {
-    sl[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    sl[32] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return 0;
-  }
+  if (!(kn > 0.f)) return 0;
   const float un = dot(u, n);
   const float target = fmaxf(S.beta_h * depth, -pr.e * un);
   const float jn = fmaxf(__fdividef(target - un, kn), 0.f);
@@ -676,9 +661,40 @@ __device__ __forceinline__ int pair_forward(const SysP& S, const BodyP* bodies, 
     const float jt = fminf(__fdividef(utn, kt), pr.mu * jn);
     J = fma3(-jt, t, J);
   }
-  sl[0] = make_float4(J.x, J.y, J.z, p.x);
-  sl[32] = make_float4(p.y, p.z, 1.f, 0.f);
+  gm.put_slot(k, lane, J, p);
+  atomicOr(gm.hit(par, pr.ba, lane), 1u << ((pr.geo >> 8) & 31));
+  atomicOr(gm.hit(par, pr.bb, lane), 1u << ((pr.geo >> 16) & 31));
   return 1;
+}
+
+// The body-body pairs this warp owns (round-robin), in two passes.  Broadphase
+// (Sec. 7.2's future work): all owned pairs' bounding spheres are tested in
+// one run of independent loads (disjoint spheres cannot touch; of the biped's
+// 120 pairs about 8 an environment pass).  Then the pairs that some
+// environment of the warp needs run their narrow phase; an environment that
+// does not need it finds no contact there.  Returns the contacts found.  Also
+// clears the body's other buffer of hit bits for the next substep: this
+// substep's first barrier has passed, so the substep before has been read, and
+// the next one sets bits only after its own first barrier.
+__device__ __forceinline__ int pairs_forward(const SysP& S, const BodyP* bodies, const PairP* pairs, int b,
+                                             GroupMem& gm, int par, int lane) {
+  *gm.hit(par ^ 1, b, lane) = 0u;
+  uint32_t near = 0;  // bit i: the i-th owned pair (at most 12: a body takes part in BRAX_MAX_BODY_PAIRS)
+  static_assert(BRAX_MAX_BODY_PAIRS / 2 <= 32, "bits of near");
+#pragma unroll 1
+  for (int k = b, i = 0; k < S.P; k += S.B, ++i) {
+    const PairP& pr = pairs[k];
+    // the centres as the bodies published them; a pair with a body that does
+    // not (several colliders) is tested before its narrow phase instead
+    const float4 ca = gm.pub4(pr.ba, 8)[lane], cb = gm.pub4(pr.bb, pr.type == kCapsuleCapsule ? 8 : 6)[lane];
+    const V3 dm = mk3(ca.x, ca.y, ca.z) - mk3(cb.x, cb.y, cb.z);
+    near |= (((pr.geo & 3) == 3 && dot(dm, dm) > pr.bound2) ? 0u : 1u) << i;
+  }
+  int counted = 0;
+#pragma unroll 1
+  for (int k = b, i = 0; k < S.P; k += S.B, ++i)
+    if (__any_sync(0xffffffffu, (near >> i) & 1u)) counted += pair_forward(S, bodies, pairs[k], gm, par, k, lane);
+  return counted;
 }
 
 // ------------------------------------------------------------------ environment layer
@@ -748,28 +764,26 @@ __device__ __forceinline__ void add_reaction(GroupMem& gm, int child, int lane, 
 // Potential integrator: v += h (F/m + g), w += h Ii tau; collision
 // integrator: the mean (or sum) of the contact velocity changes.
 template <bool kGeneral>
-__device__ __forceinline__ void integrate(const SysP& S, const BodyP& bp, GroupMem& gm, int lane, Body& s,
-                                          const Frame& f, Wrench wr, Acc acc) {
+__device__ __forceinline__ void integrate(const SysP& S, const BodyP& bp, int b, GroupMem& gm, int par, int lane,
+                                          Body& s, const Frame& f, Wrench wr, Acc acc) {
   for (int c = 0; c < bp.n_children; ++c) add_reaction(gm, bp.children[c], lane, wr);
-  for (int i = 0; kGeneral && i < bp.n_bpairs; ++i) {
-    const int code = bp.bpair[i];
-    const float4* sl = gm.slot4(code >> 1, 0) + lane;
-    const float4 c1 = sl[32];
-    if (c1.z != 0.f) {
-      const float4 c0 = sl[0];
-      const float sg = (code & 1) ? -1.f : 1.f;
-      const V3 J = sg * mk3(c0.x, c0.y, c0.z);
-      const V3 l = mk3(c0.w, c1.x, c1.y) - s.x;
-      V3 dv = bp.inv_mass * J;
-      V3 dw = mul(f.Ii, cross(l, J));
-      if (bp.flags & kAnyFrozen) {
-        dv = mask3(bp.flags, dv);
-        dw = mask3(bp.flags >> 3, dw);
-      }
-      acc.dv = acc.dv + dv;
-      acc.dw = acc.dw + dw;
-      acc.n += 1;
+  // the own pairs in contact, in pair order
+  for (uint32_t m = kGeneral && S.P > 0 ? *gm.hit(par, b, lane) : 0u; m; m &= m - 1) {
+    const int code = bp.bpair[__ffs(m) - 1];
+    V3 Ja, p;
+    gm.get_slot(code >> 1, lane, Ja, p);
+    const float sg = (code & 1) ? -1.f : 1.f;
+    const V3 J = sg * Ja;
+    const V3 l = p - s.x;
+    V3 dv = bp.inv_mass * J;
+    V3 dw = mul(f.Ii, cross(l, J));
+    if (bp.flags & kAnyFrozen) {
+      dv = mask3(bp.flags, dv);
+      dw = mask3(bp.flags >> 3, dw);
     }
+    acc.dv = acc.dv + dv;
+    acc.dw = acc.dw + dw;
+    acc.n += 1;
   }
   const float h = S.h;
   V3 v, w;

@@ -1291,10 +1291,37 @@ int64_t batch_blocks(const brax_system* s, int warps, int64_t n_envs) {
   const int64_t per = 32LL * batch_groups(s, warps);
   return (n_envs + per - 1) / per;
 }
-// The systems in the order their blocks start.
+// The default block size: the largest system's warps, or more within the same
+// launch bounds where the smaller systems then pack with fewer warp slots in
+// all (a biped of 17 warps: at 18 two quadruped groups share a block instead of
+// one).
+int batch_warps(const std::vector<const brax_system*>& sys, const std::vector<int64_t>& n_envs, int least) {
+  int most = 32, best = least;
+  for (int v : {3, 0, 1})
+    if (32 * least <= rollout_variant_max_threads(v)) {
+      most = rollout_variant_max_threads(v) / 32;
+      break;
+    }
+  int64_t fewest = -1;
+  for (int w = least; w <= most; ++w) {
+    int64_t slots = 0;
+    for (size_t i = 0; i < sys.size(); ++i) slots += batch_blocks(sys[i], w, n_envs[i]) * w;
+    if (fewest < 0 || slots < fewest) {
+      fewest = slots;
+      best = w;
+    }
+  }
+  return best;
+}
+// The systems in the order their blocks start: those with the longest substeps
+// (body-body pairs, then bodies) first, so that no long block is left for the
+// end of the launch.
 std::vector<int> batch_order(const brax_batch* b) {
   std::vector<int> order(b->sys.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    return b->sys[x]->P + b->sys[x]->B > b->sys[y]->P + b->sys[y]->B;
+  });
   return order;
 }
 }  // namespace
@@ -1318,7 +1345,7 @@ int brax_batch_create(const brax_system* const* systems, const int64_t* n_envs, 
   }
   // a block holds one group of the largest system; smaller systems pack
   // several groups of 32 environments into the same block
-  b->warps = warps;
+  b->warps = batch_warps(b->sys, b->n_envs, warps);
   *out = b;
   return BRAX_OK;
 }

@@ -1002,16 +1002,24 @@ void apply_env(const brax_system* s, Seg& sg, const EnvOut* env) {
   sg.max_z = env->p->max_z;
 }
 
-// The kernel of a system in the limb layout (0: it has none): the split kernel
-// while its warps (a quarter of the wide kernel's environments each) are at
-// most 23 an SM, 14,000 quadrupeds: there it takes 25 us a step and the wide
-// kernel 25.6; beyond, the wide kernel's warps fill the SMs (measured table at
-// rollout_limb_split_kernel).
+// The kernel of a system in the limb layout: kLimbSplit, kLimbWide or 0 (the
+// body layout), by the number of limbs and of environments.  All three give the
+// same bits.  The split kernel wins while its warps leave the SMs' schedulers
+// room; past that the wide one, except where the body layout's few warps
+// already share a short substep (one or two limbs).  Measured, us a step (split
+// / wide / body layout, default launch; 152 SMs):
+//   1 limb (pendulum)  4,096: 9.0/13.2/9.8   16,384: 12.4/13.3/10.9  32,768: 19.4/13.4/14.6  65,536: 36.5/21.0/24.0
+//   2 limbs            4,096: 6.8/18.1/13.4  16,384: 16.0/18.1/16.8  32,768: 30.4/27.8/26.9  65,536: 60.0/46.4/42.2
+//   4 (quadruped)      4,096: 9.3/16.3/18.1  12,288: 22.3/25.6/27.3  16,384: 28.7/25.8/30.2  65,536: 113/80.3/103
+//   8 limbs            2,048: 10.5/16.7/28.3  4,096: 16.8/16.9/31.5   9,752: 38.4/28.3/51.5  65,536: 249/166/325
 int limb_kind(const brax_system* s, int64_t n_envs, int n_sm) {
   if (s->n_limbs == 0 || s->pair_variant < kLimbVariant) return 0;
   if (s->pair_variant != kLimbVariant) return s->pair_variant;
   const int64_t per_warp = limb_warp_envs(s->n_limbs, true), split_warps = (n_envs + per_warp - 1) / per_warp;
-  return split_warps <= 23LL * n_sm ? kLimbSplit : kLimbWide;
+  const int most = s->n_limbs == 1 ? 4 : s->n_limbs == 2 ? 16 : s->n_limbs == 4 ? 23 : 13;  // split warps an SM
+  if (split_warps <= (int64_t)most * n_sm) return kLimbSplit;
+  if (s->n_limbs == 2 || (s->n_limbs == 1 && n_envs <= 158LL * n_sm)) return 0;
+  return kLimbWide;
 }
 
 int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, const float* state0,

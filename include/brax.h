@@ -179,7 +179,7 @@ int brax_step(const brax_system* sys, int64_t n_envs, const float* state_in, con
  * Schedule: a block keeps its environments on chip for the whole rollout,
  * so when the blocks are not a whole number of resident waves the last wave
  * would run part-empty from the first step to the last.  Then the rollout of
- * each block of environments is cut into chunks of at least 16 steps and the
+ * each block of environments is cut into chunks of at least 4 steps and the
  * launch has one block per (chunk, block of environments) item; a starting
  * block takes the next item in chunk-major order from a counter, and a chunk
  * continues from the state the previous chunk stored in state_T (so state_T

@@ -676,17 +676,18 @@ Seg make_seg(const brax_system* s, int groups, int64_t n_envs) {
 // are resident per SM, over T steps (reverse pass: T checkpoint segments).
 // Taken when the units leave the last resident wave less than 97 % full
 // (mode 1), or always (mode 2, chunks of `chunk` steps).  Mode 1 picks the
-// chunk length (at least min_chunk steps: 16, or 16 steps' worth of
+// chunk length (at least min_chunk steps: kMinChunk, or its worth of
 // segments) that minimises a round model of the launch: items run in rounds
 // of `slots` blocks in chunk-major order, a round lasts as long as its
 // longest item (a full chunk, or the shorter last chunk), and every item
-// costs a quarter step more (a new block, the state through L2, a flag
-// check).
+// costs `overhead` steps more (a new block, the state through L2, a flag
+// check): a quarter step, or kWideOverhead.
 struct SchedPlan {
   int n_chunks = 0, chunk_steps = 0;
 };
 // The plan for `slots` resident blocks (host arithmetic only).
-SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t slots, int min_chunk) {
+SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t slots, int min_chunk,
+                              double overhead = 0.25) {
   SchedPlan p;
   if (mode == 0 || T < 2 || units < 1 || slots < 1) return p;
   int64_t steps;
@@ -703,13 +704,14 @@ SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t
       const int64_t last = T - (C - 1) * len;
       const int64_t rounds = (C * units + slots - 1) / slots;
       const int64_t full = std::min(rounds, ((C - 1) * units + slots - 1) / slots);
-      const double t = (double)(full * len + (rounds - full) * last) + 0.25 * (double)(C * units) / (double)slots;
+      const double t = (double)(full * len + (rounds - full) * last) + overhead * (double)(C * units) / (double)slots;
       if (steps == 0 || t < best - 1e-9) {
         best = t;
         steps = len;
       }
     }
-    if (steps == 0) return p;
+    // no better than the static launch's part-empty last wave
+    if (steps == 0 || best >= (double)(waves * T) + overhead * (double)units / (double)slots) return p;
   }
   const int64_t C = (T + steps - 1) / steps;
   if (C < 2 || C * units > 0x3fffffff) return p;
@@ -717,11 +719,19 @@ SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t
   p.chunk_steps = (int)steps;
   return p;
 }
+// The shortest chunk, in steps: short rollouts gain from short chunks too
+// (16,384 bipeds x 50, 3.37 waves: 234 us a step in chunks of 17, 228 of 10).
+constexpr int kMinChunk = 4;
+// A chunk of the wide limb kernel costs 1.6 steps more than its steps, from
+// 65,536 quadrupeds in 8 chunks each of 25 steps (82.8 us a step) and of 50
+// (80.3).
+constexpr double kWideOverhead = 1.5;
 // per_sm() gives the resident blocks per SM.  It asks the driver (a microsecond
 // or more, of the ten that a one-step call takes), so only a launch that could
 // be cut asks: not a single step, nor a launch of at most one block an SM.
 template <class PerSm>
-SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, PerSm per_sm, int min_chunk = 16) {
+SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, PerSm per_sm,
+                        int min_chunk = kMinChunk, double overhead = 0.25) {
   if (mode == 0 || T < 2 || units < 1) return SchedPlan{};
   int n_sm = 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
@@ -731,7 +741,7 @@ SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, P
   if (mode == 1 && (units <= n_sm || T < 2 * min_chunk)) return SchedPlan{};
   const int blocks = per_sm();
   if (blocks < 1) return SchedPlan{};
-  return plan_schedule_slots(mode, chunk, units, T, (int64_t)blocks * n_sm, min_chunk);
+  return plan_schedule_slots(mode, chunk, units, T, (int64_t)blocks * n_sm, min_chunk, overhead);
 }
 
 // One region of a scheduler scratch for a launch of `units` units (null when
@@ -1070,7 +1080,8 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     apply_env(s, sg, env);
     L.seg[0] = sg;
     const SchedPlan pl =
-        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, [&] { return limb_blocks_per_sm(ll); });
+        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, [&] { return limb_blocks_per_sm(ll); }, kMinChunk,
+                      ll.split ? 0.25 : kWideOverhead);
     int64_t launch_grid;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
                                    as_stream(stream), fr);
@@ -1606,7 +1617,7 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
                                      [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, threads, smem); },
-                                     (16 + K - 1) / K);
+                                     (kMinChunk + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, fr);
   if (e == cudaSuccess)
@@ -1732,7 +1743,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   const size_t smem = shared ? pl.smem_with : pl.smem;
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
                                      [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.threads, smem); },
-                                     (16 + K - 1) / K);
+                                     (kMinChunk + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st);
   if (e == cudaSuccess)

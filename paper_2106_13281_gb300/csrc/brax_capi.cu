@@ -1065,6 +1065,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     // blocks of one warp until every SM has one, then up to four (one per
     // scheduler of an SM)
     const int64_t per_warp = limb_warp_envs(s->n_limbs, ll.split), n_warps = (n_envs + per_warp - 1) / per_warp;
+    ll.few = n_warps <= 8LL * n_sm;
     ll.warps = (int)std::min<int64_t>(kLimbMaxWarps, (n_warps + n_sm - 1) / n_sm);
     const int64_t grid = (n_warps + ll.warps - 1) / ll.warps;
     if (grid > 0x7fffffff) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout: too many environments");

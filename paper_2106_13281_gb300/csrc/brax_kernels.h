@@ -43,6 +43,7 @@ constexpr int kLimbMaxWarps = 4;
 struct LimbLaunch {
   int n_limbs, warps;
   bool frozen, split, env;
+  bool few;  // split: at most 8 warps an SM, so a thread may hold 255 registers
 };
 inline int limb_warp_envs(int n_limbs, bool split) { return (split ? 16 : 64) / n_limbs; }
 cudaError_t launch_rollout_limb(const Launch& L, const LimbLaunch& l, int grid, cudaStream_t st);

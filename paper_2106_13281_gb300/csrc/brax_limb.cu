@@ -4,12 +4,16 @@
 //
 // The arithmetic is the paired kernel's (brax_pair.cuh), operation for
 // operation and in the same order, so all three give the same bits.
+#include <cstddef>
+
 #include "brax_kernels.h"
 #include "brax_limb.cuh"
 
 namespace brax {
 
 __constant__ __align__(16) unsigned char c_pool[kPoolBytes];
+static_assert(offsetof(SysP, limb_upper) % 8 == 0 && offsetof(SysP, limb_lower) % 8 == 0 && BRAX_MAX_CHILDREN == 8,
+              "the split kernel loads the limbs' bodies as 8-byte words");
 
 namespace p2 {
 // integrate()'s potential integrator alone: the velocities before contacts.
@@ -441,12 +445,15 @@ __device__ __forceinline__ void contacts_first(const SysP2& S2, bool average, Fl
 // lasts as long as one warp takes: the wide kernel's lane does a whole limb of
 // two environments (1,260 instructions a substep), this one's a body of one
 // (560), with the contact responses in straight code beside the joint's.
-// Quadruped, us a step: up to 2,048 environments 5.7 (wide 16.4, paired 18),
-// 4,096 9.3 (16.3, 18), 8,192 14.9 (17.0, 18.6), 12,288 22.3 (25.6, 27.3),
-// 16,384 28.7 (25.8, 30.2).  Its root is computed by 2 L lanes, the wide
+// Quadruped, us a step: up to 2,048 environments 5.4 (paired 18), 4,096 9.2
+// (18), 8,192 14.8 (18), 12,288 22.2 (27), 16,384 29.2 (28).  Its root is computed by 2 L lanes, the wide
 // kernel's by L / 2 per environment, so it loses where warps fill the SMs.
-template <int L, bool kFrozen, bool kEnv>
-__global__ void __launch_bounds__(128, 3) rollout_limb_split_kernel(const __grid_constant__ Launch Ln) {
+//
+// kFew: at most 8 warps an SM, no spills (36 bytes under the 168 registers that
+// let 12 be resident, which more warps need).  With the start's loads taken
+// from the constant pool: 2,048 environments 5.9 -> 5.5 us a step.
+template <int L, bool kFrozen, bool kEnv, bool kFew>
+__global__ void __launch_bounds__(128, kFew ? 2 : 3) rollout_limb_split_kernel(const __grid_constant__ Launch Ln) {
   using namespace p2;
   using F3 = VT<float>;
   constexpr int E = 16 / L;  // environments of a warp
@@ -475,6 +482,7 @@ __global__ void __launch_bounds__(128, 3) rollout_limb_split_kernel(const __grid
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
   const SysP2& S2 = *reinterpret_cast<const SysP2*>(blob + S.pair_off);
+  const BodyP2* bodies2 = reinterpret_cast<const BodyP2*>(blob + S.pair_off + sizeof(SysP2));
   // lane-varying parameters come from the blob's copy in global memory
   const BodyP* gbodies = reinterpret_cast<const BodyP*>(sg.blob + blob_bodies_off());
   const BodyP2* gbodies2 = reinterpret_cast<const BodyP2*>(sg.blob + S.pair_off + sizeof(SysP2));
@@ -487,11 +495,13 @@ __global__ void __launch_bounds__(128, 3) rollout_limb_split_kernel(const __grid
   if (e - slot >= N) t1 = t0;  // a warp past the last environment steps nothing
   const int B = sg.B, A = sg.A, K = Ln.K;
   const int br = S.limb_root;
-  const SysP& GS = *reinterpret_cast<const SysP*>(sg.blob);
-  const int bo = level ? GS.limb_lower[limb] : GS.limb_upper[limb];
+  // the lane's body out of eight in one uniform load (a lane-varying index would
+  // cost the launch another round trip to L2)
+  const uint64_t ids = *reinterpret_cast<const uint64_t*>(level ? S.limb_lower : S.limb_upper);
+  const int bo = (int)(ids >> (8 * limb)) & 255;
   const BodyP &pr = bodies[br], &po = gbodies[bo];
   const SplitPar jp = split_par(gbodies2[bo]);
-  const SplitBody bp = split_body(gbodies2[br], pr.n_points, gbodies2[bo], po.n_points);
+  const SplitBody bp = split_body(bodies2[br], pr.n_points, gbodies2[bo], po.n_points);
   const Flags2 fl = kFrozen ? Flags2{pr.flags, po.flags} : Flags2{0u, 0u};
   const int act_idx = po.act[0];
   const bool average = S.average != 0;
@@ -649,17 +659,22 @@ __global__ void __launch_bounds__(128, 3) rollout_limb_split_kernel(const __grid
 
 // ------------------------------------------------------------------ launchers
 using LimbKernel = void (*)(const Launch);
-template <int L, bool kFrozen>
-static LimbKernel limb_kernel_f(bool split, bool env) {
-  if (split) return env ? rollout_limb_split_kernel<L, kFrozen, true> : rollout_limb_split_kernel<L, kFrozen, false>;
-  return env ? rollout_limb_kernel<L, kFrozen, true> : rollout_limb_kernel<L, kFrozen, false>;
+template <int L, bool kFrozen, bool kEnv>
+static LimbKernel limb_kernel_e(const LimbLaunch& l) {
+  if (!l.split) return rollout_limb_kernel<L, kFrozen, kEnv>;
+  return l.few ? rollout_limb_split_kernel<L, kFrozen, kEnv, true> : rollout_limb_split_kernel<L, kFrozen, kEnv, false>;
+}
+template <int L>
+static LimbKernel limb_kernel_l(const LimbLaunch& l) {
+  if (l.frozen) return l.env ? limb_kernel_e<L, true, true>(l) : limb_kernel_e<L, true, false>(l);
+  return l.env ? limb_kernel_e<L, false, true>(l) : limb_kernel_e<L, false, false>(l);
 }
 static LimbKernel limb_kernel(const LimbLaunch& l) {
   switch (l.n_limbs) {
-    case 1: return l.frozen ? limb_kernel_f<1, true>(l.split, l.env) : limb_kernel_f<1, false>(l.split, l.env);
-    case 2: return l.frozen ? limb_kernel_f<2, true>(l.split, l.env) : limb_kernel_f<2, false>(l.split, l.env);
-    case 4: return l.frozen ? limb_kernel_f<4, true>(l.split, l.env) : limb_kernel_f<4, false>(l.split, l.env);
-    default: return l.frozen ? limb_kernel_f<8, true>(l.split, l.env) : limb_kernel_f<8, false>(l.split, l.env);
+    case 1: return limb_kernel_l<1>(l);
+    case 2: return limb_kernel_l<2>(l);
+    case 4: return limb_kernel_l<4>(l);
+    default: return limb_kernel_l<8>(l);
   }
 }
 static size_t limb_smem_bytes(const LimbLaunch& l) {

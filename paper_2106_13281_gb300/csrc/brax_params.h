@@ -108,7 +108,7 @@ struct PlaneP {
   float n[3];
 };
 
-struct alignas(16) SysP {
+struct SysP {
   int32_t B, J, A, D, P, n_planes, substeps, average;
   float h, beta_h, eps;  // beta_h = baumgarte / h
   float lin_damp;        // global linear damping (1/s) of the potential integrator, 0: none
@@ -127,8 +127,10 @@ struct alignas(16) SysP {
   // Limb layout (brax_limb.cuh): n_limbs > 0 when the system is one root with
   // n_limbs limbs of two hinged bodies each, alike up to their geometry.
   int32_t n_limbs, limb_root;
-  uint8_t limb_upper[BRAX_MAX_CHILDREN], limb_lower[BRAX_MAX_CHILDREN];  // in the order of the root's children
+  alignas(8) uint8_t limb_upper[BRAX_MAX_CHILDREN];  // in the order of the root's children
+  alignas(8) uint8_t limb_lower[BRAX_MAX_CHILDREN];
 };
+static_assert(sizeof(SysP) % 16 == 0, "the bodies behind SysP start on a 16-byte boundary");
 
 // Two environments per thread (systems with hinge joints only and at most
 // two plane-contact points per body).  The floating-point parameters a warp

@@ -105,3 +105,18 @@ def test_default_launch_is_the_limb_layout_on_both_sides_of_its_rule(brax):
         other.set_pair_launch(1, 1, WIDE)
     other.rollout(*inputs(other, u, 100, 3))
     other.sync_status()
+
+
+def test_split_kernel_past_eight_warps_an_sm(brax):
+    """The split kernel's launches on both sides of its two builds (7 and 9 warps
+    an SM, 4 environments a warp)."""
+    d = S.quadruped()
+    sysm = brax(d)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    for warps in (7, 9):
+        st, a = inputs(sysm, d, 4 * warps * n_sm - 1, 6)
+        sysm.set_pair_launch(1, 1, SPLIT)
+        got = sysm.rollout(st, a, contact_count=True)
+        sysm.set_pair_launch(1, 1, 1)
+        same(got, sysm.rollout(st, a, contact_count=True))
+        sysm.sync_status()

@@ -722,9 +722,8 @@ SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t
 // The shortest chunk, in steps: short rollouts gain from short chunks too
 // (16,384 bipeds x 50, 3.37 waves: 234 us a step in chunks of 17, 228 of 10).
 constexpr int kMinChunk = 4;
-// A chunk of the wide limb kernel costs 1.6 steps more than its steps, from
-// 65,536 quadrupeds in 8 chunks each of 25 steps (82.8 us a step) and of 50
-// (80.3).
+// A chunk of the wide limb kernel costs about 1.5 steps more than its steps,
+// from 65,536 quadrupeds in chunks of 20 steps (75.2 us a step) and of 50 (72.2).
 constexpr double kWideOverhead = 1.5;
 // per_sm() gives the resident blocks per SM.  It asks the driver (a microsecond
 // or more, of the ten that a one-step call takes), so only a launch that could
@@ -877,6 +876,9 @@ int brax_system_create(const brax_desc* desc, brax_system** out) {
   if (s->n_limbs > 0) {  // the limb layout (its kernels give the paired kernel's bits)
     s->pair_mode = 1;
     s->pair_variant = kLimbVariant;
+    const BodyP* bodies = reinterpret_cast<const BodyP*>(s->blob.data() + blob_bodies_off());
+    // (the limbs are alike, so the first one tells for all)
+    s->limb_two = bodies[S->limb_upper[0]].n_points == 2 && bodies[S->limb_lower[0]].n_points == 2;
   }
   *out = s;
   return BRAX_OK;
@@ -1013,23 +1015,33 @@ void apply_env(const brax_system* s, Seg& sg, const EnvOut* env) {
 }
 
 // The kernel of a system in the limb layout: kLimbSplit, kLimbWide or 0 (the
-// body layout), by the number of limbs and of environments.  All three give the
-// same bits.  The split kernel wins while its warps leave the SMs' schedulers
-// room; past that the wide one, except where the body layout's few warps
-// already share a short substep (one or two limbs).  Measured, us a step (split
-// / wide / body layout, default launch; 152 SMs):
-//   1 limb (pendulum)  4,096: 9.0/13.2/9.8   16,384: 12.4/13.3/10.9  32,768: 19.4/13.4/14.6  65,536: 36.5/21.0/24.0
-//   2 limbs            4,096: 6.8/18.1/13.4  16,384: 16.0/18.1/16.8  32,768: 30.4/27.8/26.9  65,536: 60.0/46.4/42.2
-//   4 (quadruped)      4,096: 9.3/16.3/18.1  12,288: 22.3/25.6/27.3  16,384: 28.7/25.8/30.2  65,536: 113/80.3/103
-//   8 limbs            2,048: 10.5/16.7/28.3  4,096: 16.8/16.9/31.5   9,752: 38.4/28.3/51.5  65,536: 249/166/325
+// body layout), by the number of limbs and the split kernel's warps an SM
+// (16 / limbs environments each).  All three give the same bits.  Their time
+// rises in steps: the split kernel's with every 4 warps an SM (one more on each
+// scheduler), the wide one's with every 16 of these warps (it packs four of
+// them into one).  So the split kernel wins up to 8, the wide one up to 16,
+// where its next step lies, the split one once more up to 20.  The body layout
+// stays where its few warps share a short substep, with one limb and, for the
+// width of a step, with two.  Measured, us a step of 60 (split / wide / body
+// layout at its default launch; 152 SMs) at that many warps an SM:
+//   warps          4               7.9             11.9            15.9            18              22              33
+//   1 limb   7.6/12.6/9.8   11.6/12.7/10.9  17.1/12.7/13.0  22.3/12.9/14.6  25.2/20.4/16.8  30.3/20.6/20.3
+//   2 limbs  5.5/14.5/13.4   9.3/14.5/13.5  13.7/14.5/16.8  17.6/14.6/16.8  19.8/24.7/22.0  23.9/24.7/22.1  35.5/26.5/28.2
+//   4 limbs  5.5/13.4/18.2   9.3/13.4/18.3  13.8/13.5/18.5  17.8/13.6/18.9  20.0/22.9/26.3  24.1/23.1/26.5  35.9/24.5/30.5
+//   8 limbs  5.8/13.3/28.0   9.7/13.3/29.1  14.5/13.4/29.7  18.6/13.4/31.8  21.0/22.7/35.8  25.4/22.7/40.8  37.8/24.3/52.8
 int limb_kind(const brax_system* s, int64_t n_envs, int n_sm) {
   if (s->n_limbs == 0 || s->pair_variant < kLimbVariant) return 0;
   if (s->pair_variant != kLimbVariant) return s->pair_variant;
   const int64_t per_warp = limb_warp_envs(s->n_limbs, true), split_warps = (n_envs + per_warp - 1) / per_warp;
-  const int most = s->n_limbs == 1 ? 4 : s->n_limbs == 2 ? 16 : s->n_limbs == 4 ? 23 : 13;  // split warps an SM
-  if (split_warps <= (int64_t)most * n_sm) return kLimbSplit;
-  if (s->n_limbs == 2 || (s->n_limbs == 1 && n_envs <= 158LL * n_sm)) return 0;
-  return kLimbWide;
+  auto up_to = [&](int warps) { return split_warps <= (int64_t)warps * n_sm; };
+  if (s->n_limbs == 1) {
+    if (up_to(4)) return kLimbSplit;
+    return up_to(8) || (!up_to(16) && up_to(22)) ? 0 : kLimbWide;
+  }
+  if (up_to(s->n_limbs == 2 ? 12 : 8)) return kLimbSplit;
+  if (up_to(16)) return kLimbWide;
+  if (up_to(20)) return kLimbSplit;
+  return s->n_limbs == 2 && up_to(25) ? 0 : kLimbWide;
 }
 
 int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, const float* state0,
@@ -1062,6 +1074,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     ll.frozen = s->frozen;
     ll.env = env != nullptr;
     ll.split = kind == kLimbSplit;
+    ll.two = s->limb_two;
     // blocks of one warp until every SM has one, then up to four (one per
     // scheduler of an SM)
     const int64_t per_warp = limb_warp_envs(s->n_limbs, ll.split), n_warps = (n_envs + per_warp - 1) / per_warp;

@@ -47,6 +47,7 @@ struct brax_system {
   int pair_variant = 0;  // launch-bounds variant of the paired kernel, or kLimbVariant
   bool frozen = false;   // some body has a frozen axis
   int n_limbs = 0;       // limbs of a system in the limb layout (brax_limb.cuh), else 0
+  bool limb_two = false; // each body of the limbs has two contact points with the ground
   int bwd_variant = -1;  // launch-bounds variant of the reverse kernel (-1: smallest that fits)
   // Chunked schedule of rollouts (Sched in brax_device.cuh).  Mode 1
   // (default): used when the blocks do not fill a whole number of resident

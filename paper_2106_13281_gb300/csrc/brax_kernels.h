@@ -43,6 +43,7 @@ constexpr int kLimbMaxWarps = 4;
 struct LimbLaunch {
   int n_limbs, warps;
   bool frozen, split, env;
+  bool two;  // wide: every limb body has two contact points with the ground
   bool few;  // split: at most 8 warps an SM, so a thread may hold 255 registers
 };
 inline int limb_warp_envs(int n_limbs, bool split) { return (split ? 16 : 64) / n_limbs; }

@@ -32,14 +32,16 @@ __device__ __forceinline__ void potential(const SysP2& S2, Fl flags, const Par& 
 // The wide kernel.  What bounds it is the register file: an SM sub-partition
 // reads two 32-bit operands a cycle, so a packed multiply-add with three
 // distinct operands takes three cycles (measured: 3.0; packed multiply or add
-// 2.0; two scalar multiply-adds 3.1), and a substep's 843 packed FP32
-// instructions and about 420 others come to 2,300 of the 2,450 cycles measured
-// per warp and substep.  More resident warps therefore do not help (12 warps an
-// SM with state parked in shared memory: 88 us a step against 80), and neither
-// does a longer straight run of code.  Quadruped, 65,536 environments: 80.3 us
-// a step (816 M env-steps/s) against 84.4 of the paired kernel's best launch
-// and 103 of its default one.
-template <int L, bool kFrozen, bool kEnv>
+// 2.0; two scalar multiply-adds 3.1).  More resident warps therefore do not help
+// (12 warps an SM with state parked in shared memory: 88 us a step against 80
+// at the time), and neither does a longer straight run of code; fewer
+// instructions and a better order of them do.  Quadruped, 65,536 environments,
+// us a step: 82.3 with the lower body's contacts before the upper's and all
+// counts read in the loop; 74.4 in this order (the upper body's state is dead
+// sooner) with the counts read before it; 72.0 (910 M env-steps/s) with kTwo,
+// the two contact points of every limb body known at compile time (capsule
+// limbs).  The paired kernel: 84.9 at its best launch, 95.5 at its default one.
+template <int L, bool kFrozen, bool kEnv, bool kTwo>
 __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_constant__ Launch Ln) {
   using namespace p2;
   constexpr int E = 32 / L;  // slots of a warp; a slot is two environments
@@ -95,6 +97,9 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
   // without frozen axes every masking folds away
   const uint32_t fr_ = kFrozen ? pr.flags : 0u, fu_ = kFrozen ? pu.flags : 0u, fl_ = kFrozen ? pl.flags : 0u;
   const bool average = S.average != 0;
+  // counts the substep loop reads, held in registers
+  const int npr = pr.n_points, npu = kTwo ? 2 : pu.n_points, npl = kTwo ? 2 : pl.n_points;
+  const int nsub = S.substeps;
 
   p2::Body sr, su, sl;
   {  // chunk 0 starts from state0, a later chunk from what the previous one left in state_T
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
     if (t + 1 < t1) load_act(t + 1);
     const f2 x0 = sr.x.x;  // the root's x before the step (environment layer)
 #pragma unroll 1
-    for (int k = 0; k < S.substeps; ++k) {
+    for (int k = 0; k < nsub; ++k) {
       // the table is read anew in every substep instead of being kept in
       // registers (or spilled) across the loop
       asm volatile("" ::: "memory");
@@ -183,19 +188,19 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
       const JointOut jl = joint(ql, gl, true, p2::Pub{su.x, fu.R, su.v, su.w}, sl, fl.R, actl);
       fl.Ii = inv_inertia_world(fl.R, ql.inv_I);
       fu.Ii = inv_inertia_world(fu.R, qu.inv_I);
-      {  // lower body: contacts, integrators
-        p2::Acc acc{vzero(), vzero(), 0, 0};
-        plane_points_z(S2, ql, gl, fl_, pl.n_points, sl, fl, acc);
-        cca += acc.na;
-        ccb += acc.nb;
-        integrate(S2, average, fl_, ql, p2::Wrench{jl.F_, jl.tc}, sl, fl, acc);
-      }
       {  // upper body
         p2::Acc acc{vzero(), vzero(), 0, 0};
-        plane_points_z(S2, qu, gu, fu_, pu.n_points, su, fu, acc);
+        plane_points_z(S2, qu, gu, fu_, npu, su, fu, acc);
         cca += acc.na;
         ccb += acc.nb;
         integrate(S2, average, fu_, qu, p2::Wrench{vsub(ju.F_, jl.F_), vadd(ju.tc, jl.tp)}, su, fu, acc);
+      }
+      {  // lower body: contacts, integrators
+        p2::Acc acc{vzero(), vzero(), 0, 0};
+        plane_points_z(S2, ql, gl, fl_, npl, sl, fl, acc);
+        cca += acc.na;
+        ccb += acc.nb;
+        integrate(S2, average, fl_, ql, p2::Wrench{jl.F_, jl.tc}, sl, fl, acc);
       }
       {  // root: the limbs' reactions in child order, alike on all its lanes
         p2::Wrench wr{vzero(), vzero()};
@@ -217,7 +222,7 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
         }
         fr.Ii = inv_inertia_world(fr.R, qr.inv_I);
         p2::Acc acc{vzero(), vzero(), 0, 0};
-        plane_points_z(S2, qr, qr, fr_, pr.n_points, sr, fr, acc);
+        plane_points_z(S2, qr, qr, fr_, npr, sr, fr, acc);
         if (limb == 0) {
           cca += acc.na;
           ccb += acc.nb;
@@ -661,7 +666,7 @@ __global__ void __launch_bounds__(128, kFew ? 2 : 3) rollout_limb_split_kernel(c
 using LimbKernel = void (*)(const Launch);
 template <int L, bool kFrozen, bool kEnv>
 static LimbKernel limb_kernel_e(const LimbLaunch& l) {
-  if (!l.split) return rollout_limb_kernel<L, kFrozen, kEnv>;
+  if (!l.split) return l.two ? rollout_limb_kernel<L, kFrozen, kEnv, true> : rollout_limb_kernel<L, kFrozen, kEnv, false>;
   return l.few ? rollout_limb_split_kernel<L, kFrozen, kEnv, true> : rollout_limb_split_kernel<L, kFrozen, kEnv, false>;
 }
 template <int L>

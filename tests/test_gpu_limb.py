@@ -107,6 +107,43 @@ def test_default_launch_is_the_limb_layout_on_both_sides_of_its_rule(brax):
     other.sync_status()
 
 
+def ball_limbs(no_lower):
+    """Two limbs whose lower bodies carry one point (a ball) or none."""
+    sb = S.SceneBuilder()
+    t = sb.body("torso", 10.0, S.UNIT_INERTIA, (0, 0, 0.75))
+    sb.collider(t, S.CAPSULE, radius=0.25, length=0.5)
+    ground = sb.plane()
+    sb.pair(sb.collider_of(t), ground)
+    for k, x in enumerate((-1.0, 1.0)):
+        d = np.array([x, 0.0, 0.0])
+        hip = np.array([0, 0, 0.75]) + 0.25 * d
+        th = sb.capsule_body(f"thigh{k}", 1.0, 0.08, 0.4, hip + 0.2 * d, d, inertia=S.UNIT_INERTIA)
+        sh = sb.body(f"foot{k}", 1.0, S.UNIT_INERTIA, hip + 0.5 * d)
+        sb.collider(sh, S.CAPSULE, radius=0.1, length=0.2)
+        jh = sb.joint(t, th, hip, axis=np.array([0.0, 1, 0]), ref=d, limits=((-40, 40),), **S.QUADRUPED_JOINT)
+        sb.joint(th, sh, hip + 0.4 * d, axis=np.array([0.0, 1, 0]), ref=d, limits=((-40, 40),), **S.QUADRUPED_JOINT)
+        sb.actuator(jh, 0, 100.0)
+        sb.pair(sb.collider_of(th), ground)
+        if not no_lower:
+            sb.pair(sb.collider_of(sh), ground)
+    return sb.build()
+
+
+@pytest.mark.parametrize("no_lower", [False, True])
+def test_limbs_with_other_point_counts(brax, no_lower):
+    """Lower bodies of one point and of none: the wide kernel's counts at run time."""
+    d = ball_limbs(no_lower)
+    sysm = brax(d)
+    st, a = inputs(sysm, d, 333, 40)
+    sysm.set_pair_launch(1, 1, 1)
+    ref = sysm.rollout(st, a, K=7, checkpoints=True, torso=True, contact_count=True)
+    assert int(ref["contact_count"].sum()) > 0
+    for v in (WIDE, SPLIT):
+        sysm.set_pair_launch(1, 1, v)
+        same(sysm.rollout(st, a, K=7, checkpoints=True, torso=True, contact_count=True), ref)
+        sysm.sync_status()
+
+
 def test_split_kernel_past_eight_warps_an_sm(brax):
     """The split kernel's launches on both sides of its two builds (7 and 9 warps
     an SM, 4 environments a warp)."""

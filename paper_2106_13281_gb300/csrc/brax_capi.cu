@@ -1605,7 +1605,7 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
   std::memset(&L, 0, sizeof(L));
   L.n_segs = 1;
   L.T = T;
-  L.K = K;  // segment boundaries follow the checkpoints written with K
+  L.K = Ke;  // segment boundaries follow the checkpoints; the workspace's layout is Ke's
   Seg sg = make_seg(s, 1, n_envs);
   const int64_t grid = bwd_groups_total(n_envs);
   if (grid > 0x7fffffff) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout_backward: too many environments");
@@ -1730,7 +1730,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   std::memset(&L, 0, sizeof(L));
   L.n_segs = (int)b->sys.size();
   L.T = T;
-  L.K = K;
+  L.K = std::min(K, T);  // the workspace's layout (one segment when K >= T)
   int cta = 0;
   for (int j = 0; j < L.n_segs; ++j) {
     const int i = pl.order[j];

@@ -331,6 +331,10 @@ int brax_batch_offsets(const brax_batch* batch, int32_t T, int32_t K, int32_t i,
  * environments were waited for). */
 int brax_batch_rollout(const brax_batch* batch, int32_t T, int32_t K, const float* state0, const float* actions,
                        float* state_T, float* checkpoints, float* torso_traj, void* stream);
+/* The size covers, up to 1 GiB, every substep state of a checkpoint segment
+ * (K x substeps per environment).  brax_batch_rollout_backward also takes a
+ * smaller workspace, down to K + substeps states, and then recomputes each
+ * step's substeps; the gradients are the same bits. */
 int brax_batch_workspace_size(const brax_batch* batch, int32_t T, int32_t K, size_t* bytes);
 int brax_batch_rollout_backward(const brax_batch* batch, int32_t T, int32_t K, const float* state0,
                                 const float* actions, const float* checkpoints, const float* g_state_T,

@@ -47,7 +47,8 @@ __host__ __device__ inline int bwd_fwd_floats(int B, int P, bool slots_in_smem) 
 }
 __host__ __device__ inline int bwd_group_floats(int B, int P) { return bwd_fwd_floats(B, P, false) + bwd_extra_floats(B, P); }
 // Workspace of one group: step states [K][13][B][32], substep states
-// [S][13][B][32], pair slots [P][kSlotFields][32], pair adjoints
+// [S][13][B][32] (Launch::keep: no step states, a whole segment's substep
+// states, so K = 0 and S = K x substeps below), pair slots [P][kSlotFields][32], pair adjoints
 // [P][2][18][32], and the state adjoint carried from one chunk of a chunked
 // schedule to the next [13][B][32].
 __host__ __device__ inline int64_t ws_pairg_off(int B, int P, int K, int S) {
@@ -463,7 +464,15 @@ __device__ __forceinline__ void bwd_substep_iso(const SysP& S, const PlaneP* pla
 // schedule (Sched; chunk_steps counts segments, chunk 0 holds the last
 // ones), one chunk of the unit of the item it takes; the state adjoint then
 // passes from chunk to chunk through the workspace.
-template <bool kGeneral, bool kIso, bool kShared>
+//
+// Launch::keep: the segment's forward pass stores every substep state instead
+// of every step state, so that the way back needs no second forward pass:
+// (K - 1)(substeps - 1) substeps a segment fewer.  Four scenes of 8,192
+// environments, T = 8, K = 4: 8.75 -> 7.68 ms; pendulum and quadruped, 2,730
+// each: 0.387 -> 0.326.  The general kernel takes either; the hinge-only ones
+// are built for each (kKeep), since the choice at run time cost the other
+// layout 1.5 % (65,536 quadrupeds, K = 1).
+template <bool kGeneral, bool kIso, bool kShared, bool kKeep>
 __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -513,20 +522,23 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   float* gbase = reinterpret_cast<float*>(smem) + g * bwd_group_floats(B, P);
   GroupMem gm = group_mem(gbase, B, 0);
   const int K = L.K, T = L.T, nsub = S.substeps;
-  float* ws = sg.ws + group * ws_group_floats(B, P, K, nsub);
-  if (kGeneral) gm.slot = reinterpret_cast<float2*>(ws + (int64_t)(K + nsub) * 13 * B * 32);  // pair impulses live in the workspace
+  // step and substep states a group's workspace holds
+  const bool keep = kGeneral ? L.keep != 0 : kKeep;
+  const int Kw = keep ? 0 : K, Sw = keep ? K * nsub : nsub;
+  float* ws = sg.ws + group * ws_group_floats(B, P, Kw, Sw);
+  if (kGeneral) gm.slot = reinterpret_cast<float2*>(ws + (int64_t)(Kw + Sw) * 13 * B * 32);  // pair impulses live in the workspace
   BwdMem bm;
   bm.gwr = gbase + bwd_fwd_floats(B, P, false);
   bm.gpub = bm.gwr + B * 6 * 32;
   bm.gacc = bm.gpub + B * 18 * 32;
-  bm.pairg = ws + ws_pairg_off(B, P, K, nsub);
+  bm.pairg = ws + ws_pairg_off(B, P, Kw, Sw);
   int par = 0;  // which buffer of hit bits the substep uses; both start clear
   if (kGeneral) *gm.hit(0, b, lane) = *gm.hit(1, b, lane) = 0u;
   const int bar = 1 + g, nthr = 32 * B;
   const BodyP& bp = bodies[b];
   const int stride = B * 32;
   float* ws_steps = ws + b * 32 + lane;
-  float* ws_subs = ws + (int64_t)K * 13 * B * 32 + b * 32 + lane;
+  float* const ws_subs0 = ws + (int64_t)Kw * 13 * B * 32 + b * 32 + lane;
 
   HingeRegs hr;
   PointRegs pr[2];
@@ -541,7 +553,7 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   GBody gs = zero_gbody();
   if (c > 0) {  // L2 loads: the previous chunk may have run on another SM
     // the adjoint carried between chunks (lane-contiguous, like the step states)
-    const float* carry = ws_steps + ws_carry_off(B, P, K, nsub);
+    const float* carry = ws_steps + ws_carry_off(B, P, Kw, Sw);
     float v[13];
 #pragma unroll
     for (int i = 0; i < 13; ++i) v[i] = __ldcg(carry + i * stride);
@@ -585,24 +597,34 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
       s.v = zero3();
       s.w = zero3();
     }
-    // recompute the segment's step states
+    // recompute the segment's step states, or (keep) all its substep states
     for (int t = t0; t < t1; ++t) {
-      store_body_ws(ws_steps + (int64_t)(t - t0) * 13 * stride, stride, s);
-      if (t + 1 < t1) {
+      if (!keep) store_body_ws(ws_steps + (int64_t)(t - t0) * 13 * stride, stride, s);
+      if (keep || t + 1 < t1) {
         load_act(t);
-        for (int k = 0; k < nsub; ++k)
+        float* sub = ws_subs0 + (int64_t)(t - t0) * nsub * 13 * stride;
+        for (int k = 0; k < nsub; ++k) {
+          if (keep) {
+            store_body_ws(sub, stride, s);
+            sub += 13 * stride;
+            if (t + 1 == t1 && k + 1 == nsub) break;
+          }
           fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, par ^= 1, s, act);
+        }
       }
     }
     for (int t = t1 - 1; t >= t0; --t) {
-      load_body_ws(ws_steps + (int64_t)(t - t0) * 13 * stride, stride, s);
+      float* const ws_subs = ws_subs0 + (keep ? (int64_t)(t - t0) * nsub * 13 * stride : 0);
       load_act(t);
-      __syncwarp();
-      discard_state_ws(ws_steps - lane + (int64_t)(t - t0) * 13 * stride, stride, lane);
-      for (int k = 0; k < nsub; ++k) {
-        store_body_ws(ws_subs + (int64_t)k * 13 * stride, stride, s);
-        if (k + 1 < nsub)
-          fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, par ^= 1, s, act);
+      if (!keep) {
+        load_body_ws(ws_steps + (int64_t)(t - t0) * 13 * stride, stride, s);
+        __syncwarp();
+        discard_state_ws(ws_steps - lane + (int64_t)(t - t0) * 13 * stride, stride, lane);
+        for (int k = 0; k < nsub; ++k) {
+          store_body_ws(ws_subs + (int64_t)k * 13 * stride, stride, s);
+          if (k + 1 < nsub)
+            fwd_substep<kGeneral, kIso>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, par ^= 1, s, act);
+        }
       }
       if (sg.g_torso && b == 0 && valid) {
         const float* gt = sg.g_torso + ((int64_t)t * N + env) * 3;
@@ -629,7 +651,7 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
     }
   }
   if (seg_lo > 0) {  // not the first segments yet: hand the adjoint to the next chunk
-    float* carry = ws_steps + ws_carry_off(B, P, K, nsub);
+    float* carry = ws_steps + ws_carry_off(B, P, Kw, Sw);
     const float v[13] = {gs.x.x, gs.x.y, gs.x.z, gs.q[0], gs.q[1], gs.q[2], gs.q[3],
                          gs.v.x, gs.v.y, gs.v.z, gs.w.x, gs.w.y, gs.w.z};
 #pragma unroll
@@ -662,33 +684,36 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
 // groups per SM), which holds more of the adjoint's live values than the
 // 96 registers (576, 1) gives.  Each is compiled for three kinds of system:
 // hinge-only, hinge-only with isotropic inertia (bwd_substep_iso), general.
-template <int MAXT, int MINB, bool kGeneral, bool kIso, bool kShared>
+template <int MAXT, int MINB, bool kGeneral, bool kIso, bool kShared, bool kKeep>
 __global__ void __launch_bounds__(MAXT, MINB) rollout_bwd_kernel(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso, kShared>(L);
+  rollout_bwd_body<kGeneral, kIso, kShared, kKeep>(L);
 }
-template <bool kGeneral, bool kIso, bool kShared>
+template <bool kGeneral, bool kIso, bool kShared, bool kKeep>
 __global__ void __maxnreg__(112) rollout_bwd_kernel_r112(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso, kShared>(L);
+  rollout_bwd_body<kGeneral, kIso, kShared, kKeep>(L);
 }
 
 using BwdKernel = void (*)(const Launch);
-template <bool G, bool I, bool Sh>
+template <bool G, bool I, bool Sh, bool Kp>
 static BwdKernel bwd_kernel_t(int variant) {
   switch (variant) {
-    case 0: return rollout_bwd_kernel<384, 2, G, I, Sh>;
-    case 1: return rollout_bwd_kernel<576, 1, G, I, Sh>;
-    case 3: return rollout_bwd_kernel<288, 3, G, I, Sh>;
-    case 4: return rollout_bwd_kernel_r112<G, I, Sh>;
-    default: return rollout_bwd_kernel<1024, 1, G, I, Sh>;
+    case 0: return rollout_bwd_kernel<384, 2, G, I, Sh, Kp>;
+    case 1: return rollout_bwd_kernel<576, 1, G, I, Sh, Kp>;
+    case 3: return rollout_bwd_kernel<288, 3, G, I, Sh, Kp>;
+    case 4: return rollout_bwd_kernel_r112<G, I, Sh, Kp>;
+    default: return rollout_bwd_kernel<1024, 1, G, I, Sh, Kp>;
   }
 }
-static BwdKernel bwd_kernel(int variant, bool general, bool iso, bool shared) {
-  if (general) return shared ? bwd_kernel_t<true, false, true>(variant) : bwd_kernel_t<true, false, false>(variant);
-  return iso ? bwd_kernel_t<false, true, false>(variant) : bwd_kernel_t<false, false, false>(variant);
+static BwdKernel bwd_kernel(int variant, bool general, bool iso, bool shared, bool keep) {
+  if (general)
+    return shared ? bwd_kernel_t<true, false, true, false>(variant) : bwd_kernel_t<true, false, false, false>(variant);
+  if (keep)
+    return iso ? bwd_kernel_t<false, true, false, true>(variant) : bwd_kernel_t<false, false, false, true>(variant);
+  return iso ? bwd_kernel_t<false, true, false, false>(variant) : bwd_kernel_t<false, false, false, false>(variant);
 }
 
-int backward_blocks_per_sm(int variant, bool general, bool iso, bool shared, int threads, size_t smem) {
-  const BwdKernel k = bwd_kernel(variant, general, iso, shared);
+int backward_blocks_per_sm(int variant, bool general, bool iso, bool shared, bool keep, int threads, size_t smem) {
+  const BwdKernel k = bwd_kernel(variant, general, iso, shared, keep);
   if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
@@ -702,7 +727,7 @@ int backward_variant_max_threads(int variant) {
 
 cudaError_t launch_rollout_backward(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,
                                     bool iso, bool shared, cudaStream_t st) {
-  const BwdKernel k = bwd_kernel(variant, general, iso, shared);
+  const BwdKernel k = bwd_kernel(variant, general, iso, shared, L.keep != 0);
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, threads, smem, st>>>(L);

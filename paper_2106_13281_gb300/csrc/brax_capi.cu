@@ -1630,7 +1630,7 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
   if (shared) smem += param_smem(s);
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
-                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, threads, smem); },
+                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, false, threads, smem); },
                                      (kMinChunk + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, fr);
@@ -1672,9 +1672,16 @@ struct BwdBatchPlan {
   std::vector<int> groups, blocks;  // by system
   std::vector<int> order;           // the systems as their blocks start
   std::vector<size_t> ws_off;
+  bool keep = false;  // every substep state of a segment in the workspace
 };
-BwdBatchPlan plan_batch_backward(const brax_batch* b, int32_t K) {
+// The most workspace that keeping a segment's substep states may take.  Beyond
+// it (or when the caller's workspace holds no more) the reverse kernel keeps the
+// K step states and recomputes each step's substeps before it goes back over
+// them: K (substeps - 1) more forward substeps a segment.
+constexpr size_t kKeepBytes = size_t(1) << 30;
+BwdBatchPlan plan_batch_layout(const brax_batch* b, int32_t K, bool keep) {
   BwdBatchPlan pl;
+  pl.keep = keep;
   pl.threads = 32 * b->warps;
   pl.order = batch_order(b);
   for (size_t i = 0; i < b->sys.size(); ++i) {
@@ -1686,7 +1693,9 @@ BwdBatchPlan plan_batch_backward(const brax_batch* b, int32_t K) {
     pl.blocks.push_back(nb);
     pl.grid += nb;
     pl.ws_off.push_back(pl.ws_bytes);
-    const size_t wb = (size_t)nb * G * (size_t)backward_ws_floats_per_group(s->B, s->P, K, S->substeps) * sizeof(float);
+    const size_t wb = (size_t)nb * G *
+                      (size_t)backward_ws_floats_per_group(s->B, s->P, keep ? 0 : K, keep ? K * S->substeps : S->substeps) *
+                      sizeof(float);
     pl.ws_bytes += (wb + 255) & ~size_t(255);
     pl.smem = std::max(pl.smem, backward_smem_bytes(s->B, s->P, G));
     pl.smem_with = std::max(pl.smem_with, backward_smem_bytes(s->B, s->P, G) + param_smem(s));
@@ -1694,6 +1703,13 @@ BwdBatchPlan plan_batch_backward(const brax_batch* b, int32_t K) {
     pl.iso = pl.iso && s->iso;
   }
   return pl;
+}
+BwdBatchPlan plan_batch_backward(const brax_batch* b, int32_t K, size_t limit = kKeepBytes) {
+  if (K > 1 && K <= 4096) {
+    BwdBatchPlan pl = plan_batch_layout(b, K, true);
+    if (pl.ws_bytes <= std::min(limit, kKeepBytes)) return pl;
+  }
+  return plan_batch_layout(b, K, false);
 }
 }  // namespace
 
@@ -1720,7 +1736,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
     return BRAX_OK;
   }
   if (!state0 || !checkpoints) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_batch_rollout_backward: null inputs");
-  const BwdBatchPlan pl = plan_batch_backward(b, std::min(K, T));
+  const BwdBatchPlan pl = plan_batch_backward(b, std::min(K, T), workspace_bytes);
   if (!workspace || workspace_bytes < pl.ws_bytes)
     return fail(BRAX_ERR_WORKSPACE, "brax_batch_rollout_backward: workspace missing or too small");
   if (reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
@@ -1731,6 +1747,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   L.n_segs = (int)b->sys.size();
   L.T = T;
   L.K = std::min(K, T);  // the workspace's layout (one segment when K >= T)
+  L.keep = pl.keep ? 1 : 0;
   int cta = 0;
   for (int j = 0; j < L.n_segs; ++j) {
     const int i = pl.order[j];
@@ -1756,7 +1773,7 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   const bool shared = pl.general && fits_block(pl.smem_with, device);
   const size_t smem = shared ? pl.smem_with : pl.smem;
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
-                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.threads, smem); },
+                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.keep, pl.threads, smem); },
                                      (kMinChunk + K - 1) / K);
   int64_t launch_grid;
   cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st);

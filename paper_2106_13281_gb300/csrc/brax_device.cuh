@@ -76,7 +76,7 @@ struct Sched {
 struct Launch {
   int32_t n_segs;
   int32_t T, K;
-  int32_t pad;
+  int32_t keep;  // reverse: the workspace holds a segment's substep states (K x substeps of them)
   Seg seg[BRAX_MAX_SEGS];
   Sched sc;
 };

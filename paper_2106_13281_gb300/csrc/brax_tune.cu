@@ -4,7 +4,8 @@
 // Forward candidates: the one-environment kernel with 1..4 groups of 32
 // environments per block under each launch-bounds variant that admits the
 // block, and, for systems that have it, the two-environments kernel with
-// 1..4 groups of 64.  Reverse candidates: checkpoint intervals K from
+// 1..4 groups of 64 and, where the system has one, the limb layout.  Reverse
+// candidates: checkpoint intervals K from
 // {1, 2, 4, 5, 8, 10, 16, 20, 25, 50, 100} (K <= T, checkpoints + workspace
 // within the memory budget) times the reverse kernel's launch-bounds
 // variants; the figure compared is (forward with checkpoints + reverse) per

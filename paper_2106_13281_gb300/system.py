@@ -71,7 +71,10 @@ class BraxSystem:
     def set_pair_launch(self, mode: int, groups: int = 1, variant: int = 0):
         """Two-environments-per-thread kernel of hinge-only systems: mode 1
         uses it for rollout/step (groups of 64 environments per block), mode 0
-        falls back to the one-environment kernel."""
+        falls back to the one-environment kernel.  Variants 5 to 7 (systems of
+        one root and limbs of two hinged bodies): the limb layout, the kernel
+        picked by size (the default of such a system), the wide or the split
+        one."""
         check(self._L.brax_system_set_pair_launch(self._h, mode, groups, variant))
 
     def set_schedule(self, mode: int, chunk_steps: int = 0, first_item: int = 0, wait_ns: int = 2_000_000_000):

@@ -50,7 +50,7 @@ def test_reverse_pass_stays_inside_its_workspace(systems, T, K):
 
 def batch_of(systems, T, K):
     from paper_2106_13281_gb300.system import BraxBatch
-    n = [40, 70, 33]
+    n = [40, 70, 33][:len(systems)]
     b = BraxBatch(systems, n)
     parts = [inputs(s, m, T) for s, m in zip(systems, n)]
     st, a = torch.cat([p[0].flatten() for p in parts]), torch.cat([p[1].flatten() for p in parts])
@@ -66,3 +66,27 @@ def test_batch_reverse_pass_stays_inside_its_workspace(systems, T, K):
     for s in systems:
         s.sync_status()
     assert bool((big[need:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("names", [("pendulum", "quadruped"), ("quadruped", "biped")])
+@pytest.mark.parametrize("T,K", [(5, 2), (4, 4)])
+def test_batch_gradients_do_not_depend_on_the_workspace(systems, names, T, K):
+    """The size asked for (all substep states of a segment) and a smaller one
+    (step states, substeps recomputed): the same bits, for hinge-only systems
+    and for general ones; less still is refused."""
+    from paper_2106_13281_gb300.binding import _ptr, _stream
+    sub = [s for s, n in zip(systems, NAMES) if n in names]
+    b, st, a, ck = batch_of(sub, T, K)
+    need = b.workspace_size(T, K)
+    g = torch.ones_like(st)
+    outs = []
+    for nbytes in (need, need - 1):
+        ws, big = guarded(nbytes)
+        ga, gs = torch.empty_like(a), torch.empty_like(st)
+        args = (b._h, T, K, _ptr(st), _ptr(a), _ptr(ck), _ptr(g), None, _ptr(ga), _ptr(gs), _ptr(ws))
+        assert b._L.brax_batch_rollout_backward(*args, nbytes, _stream()) == 0
+        torch.cuda.synchronize()
+        assert bool((big[nbytes:] == 0xA5).all())
+        outs.append((ga, gs))
+        assert b._L.brax_batch_rollout_backward(*args, 4096, _stream()) == 7
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])

@@ -63,12 +63,13 @@ struct Rejected {
     if (!(cond)) throw Rejected{std::string(msg)}; \
   } while (0)
 
-// Validate a descriptor and flatten it into the parameter blob.
 // Whether the system has the limb layout's shape (brax_limb.cuh), and which
-// body is which: one root whose L children (L a power of two) each have one
-// child of their own and nothing else, every body of at most two plane points
-// on z-up ground, and all upper (and all lower) bodies alike but for their
-// geometry (offsets, frames, point positions).
+// body is which: one root, body 0 (the body of the torso path and of the
+// environment layer, which the limb kernels take from the root's lanes), whose
+// L children (L a power of two) each have one child of their own and nothing
+// else, every body of at most two plane points on z-up ground, and all upper
+// (and all lower) bodies alike but for their geometry (offsets, frames, point
+// positions).
 void find_limbs(SysP& S, const std::vector<BodyP>& bodies, const std::vector<PlaneP>& planes) {
   S.n_limbs = 0;
   int root = -1;
@@ -77,7 +78,7 @@ void find_limbs(SysP& S, const std::vector<BodyP>& bodies, const std::vector<Pla
       if (root >= 0) return;
       root = b;
     }
-  if (root < 0 || !S.flat) return;
+  if (root != 0 || !S.flat) return;
   const BodyP& r = bodies[root];
   const int L = r.n_children;
   if (L < 1 || L > BRAX_MAX_CHILDREN || (L & (L - 1)) || S.B != 1 + 2 * L) return;
@@ -106,6 +107,7 @@ void find_limbs(SysP& S, const std::vector<BodyP>& bodies, const std::vector<Pla
   S.n_limbs = L;
 }
 
+// Validate a descriptor and flatten it into the parameter blob.
 std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int* P_out) {
   REQUIRE(d.version == 1 || d.version == BRAX_DESC_VERSION, "version: expected 1 or BRAX_DESC_VERSION");
   // a version-1 descriptor ends before the variant fields: they are off

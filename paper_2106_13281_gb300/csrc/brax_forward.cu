@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
 #pragma unroll
       for (int a = 0; a < 3; ++a) act[a] = bp.act[a] >= 0 ? __ldg(ap + bp.act[a]) : 0.f;
     }
-    if (kEnv && b == 0) gm.react4(0, 0)[lane].x = s.x.x;  // the root's x before the step (its react slot is free)
+    // body 0's x before the step, where the contact count of a plain rollout lies
+    if (kEnv && b == 0) gm.cnt[lane] = __float_as_int(s.x.x);
     for (int k = 0; k < nsub; ++k)
       ccount += substep_forward<kGeneral>(S, bodies, pairs, planes, bp, hr, pr, b, B, lane, gm, bar, nthr, tree,
                                           par ^= 1, s, act);
@@ -226,11 +227,11 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
       }
       if (b == 0) {
         float ctrl = 0.f;
-        for (int c = 1; c < B; ++c)
+        for (int c = 0; c < B; ++c)
           if (bodies[c].flags & kHasParent) ctrl += gm.pub4(c, 4)[lane].z;
         bool done = false;
         if (valid)
-          done = root_env(sg, s, gm.react4(0, 0)[lane].x, ctrl, ob, sg.reward + (int64_t)t * N + env,
+          done = root_env(sg, s, __int_as_float(gm.cnt[lane]), ctrl, ob, sg.reward + (int64_t)t * N + env,
                           sg.done + (int64_t)t * N + env);
         gm.react4(0, 0)[lane].y = done ? 1.f : 0.f;
       }
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_pair_kernel(const __grid_c
       const float* ap = sg.actions + (int64_t)t * N * A + act_idx;
       act = make_float2(va ? __ldg(ap + ea * A) : 0.f, vb ? __ldg(ap + eb * A) : 0.f);
     }
-    if (kEnv && b == 0) gm.reactf(0, 10)[lane] = s.x.x;  // the root's x before the step (its react slot is free)
+    if (kEnv && b == 0) gm.reactf(0, 10)[lane] = s.x.x;  // body 0's x before the step, in a free react field
     for (int k = 0; k < nsub; ++k) {
       kinematic(S2, bp.flags, s);
       p2::Frame f;
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_pair_kernel(const __grid_c
         }
         if (b == 0) {
           float ctrl = 0.f;
-          for (int cb = 1; cb < B; ++cb)
+          for (int cb = 0; cb < B; ++cb)
             if (bodies[cb].flags & kHasParent) ctrl += c(gm.reactf(cb, 9)[lane]);
           bool done = false;
           if (vh)

@@ -66,3 +66,40 @@ def test_torso_and_environment_follow_body_0(brax, name, drop, N):
     for k in ref:
         assert torch.equal(got[k], ref[k]), k
     default.sync_status()
+
+
+@pytest.mark.parametrize("name,drop", [("quadruped", 0.38), ("biped", 0.0)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_environment_layer_of_a_jointed_body_0(brax, name, drop, mode):
+    """Body 0 as a joint's child (it has a parent and an actuator of its own):
+    observation, reward and done of each step against the oracle's formulas on
+    the GPU's own states, in the one-environment kernels and in the default
+    launch, with the tolerances of test_gpu_env.py."""
+    from oracle import env as oenv
+    d = S.SCENES[name]()
+    r, order = root_last(d)
+    N, T = 70, 4
+    st, a = inputs(brax, d, order, N, T, drop)
+    sysm = brax(r)
+    if mode == 0 and sysm.paired:
+        sysm.set_pair_launch(0, 1, 0)
+    z = st[:, 0, 2].cpu().numpy()
+    lo, hi = np.float32(np.quantile(z, 0.3)), np.float32(10.0)
+    spec = dict(forward_weight=1.25, healthy_reward=0.5, ctrl_cost=0.3, min_z=float(lo), max_z=float(hi))
+    for t in range(T):
+        out = sysm.env_rollout(st, a[t:t + 1], auto_reset=False, **spec)
+        s0, s1 = st.cpu().numpy().astype(np.float64), out["state_T"].cpu().numpy().astype(np.float64)
+        obs, rew = out["obs"].cpu().numpy()[0], out["reward"].cpu().numpy()[0]
+        z = s1[:, 0, 2].astype(np.float32)
+        done = (z < lo) | (z > hi)
+        assert np.array_equal(out["done"].cpu().numpy()[0].astype(bool), done)
+        ref = oenv.observe(r, s1)
+        nd = (ref.shape[1] - 11) // 2
+        assert np.array_equal(obs[:, :11], ref[:, :11])
+        assert np.abs(obs[:, 11:11 + nd] - ref[:, 11:11 + nd]).max() < 2e-5
+        assert (np.abs(obs[:, 11 + nd:] - ref[:, 11 + nd:]) <= 1e-5 * (1.0 + np.abs(ref[:, 11 + nd:]))).all()
+        ctrl = np.sum(np.clip(a[t].cpu().numpy().astype(np.float64), -1, 1) ** 2, axis=1)
+        exp = 1.25 * (s1[:, 0, 0] - s0[:, 0, 0]) / r["dt"] + 0.5 * ~done - 0.3 * ctrl
+        assert np.abs(rew - exp).max() < 1e-5 * (1.0 + np.abs(exp).max())
+        st = out["state_T"]
+    sysm.sync_status()

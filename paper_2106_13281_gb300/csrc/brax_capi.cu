@@ -1326,10 +1326,20 @@ int64_t batch_blocks(const brax_system* s, int warps, int64_t n_envs) {
   const int64_t per = 32LL * batch_groups(s, warps);
   return (n_envs + per - 1) / per;
 }
+// Shared memory of a batch's largest block at `warps` warps, forward or
+// reverse, with the parameters (bytes).
+size_t batch_smem(const std::vector<const brax_system*>& sys, int warps) {
+  size_t most = 0;
+  for (const brax_system* s : sys) {
+    const int G = batch_groups(s, warps);
+    most = std::max(most, std::max(G * group_bytes(s), backward_smem_bytes(s->B, s->P, G)) + param_smem(s));
+  }
+  return most;
+}
 // The default block size: the largest system's warps, or more within the same
-// launch bounds where the smaller systems then pack with fewer warp slots in
-// all (a biped of 17 warps: at 18 two quadruped groups share a block instead of
-// one).
+// launch bounds and a block's shared memory where the smaller systems then pack
+// with fewer warp slots in all (a biped of 17 warps: at 18 two quadruped groups
+// share a block instead of one).
 int batch_warps(const std::vector<const brax_system*>& sys, const std::vector<int64_t>& n_envs, int least) {
   int most = 32, best = least;
   for (int v : {3, 0, 1})
@@ -1339,6 +1349,7 @@ int batch_warps(const std::vector<const brax_system*>& sys, const std::vector<in
     }
   int64_t fewest = -1;
   for (int w = least; w <= most; ++w) {
+    if (w > least && !fits_block(batch_smem(sys, w), sys[0]->device)) continue;
     int64_t slots = 0;
     for (size_t i = 0; i < sys.size(); ++i) slots += batch_blocks(sys[i], w, n_envs[i]) * w;
     if (fewest < 0 || slots < fewest) {

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
         integrate(S2, average, fr_, qr, wr, sr, fr, acc);
       }
     }
-    if (sg.torso && limb == 0) {  // the root is body 0
+    if (sg.torso && br == 0 && limb == 0) {
       float* tp = sg.torso + (int64_t)t * N * 3;
       if (va) {
         tp[ea * 3 + 0] = sr.x.x.x;
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(128, kFew ? 2 : 3) rollout_limb_split_kernel(c
       s.v = vfma(inv, dv, nv);
       s.w = vfma(inv, dw, nw);
     }
-    if (sg.torso && root_lane && valid) {  // the root is body 0
+    if (sg.torso && br == 0 && root_lane && valid) {
       float* tp = sg.torso + ((int64_t)t * N + e) * 3;
       tp[0] = s.x.x.x;
       tp[1] = s.x.y.x;

@@ -188,13 +188,15 @@ int brax_step(const brax_system* sys, int64_t n_envs, const float* state_in, con
  * static schedule.  The flags and the counter live in scratch the system
  * owns: four regions used in turn by successive chunked launches of the
  * system (forward and reverse), each zeroed on the launch's stream when it is
- * taken.  So at most four chunked launches of one system may be in flight on
- * the GPU at once: a fifth (on another stream), or an eager launch between
- * replays of a captured CUDA graph that holds one of the regions, can zero a
- * region a running kernel still uses and silently corrupt its results.  The
- * first call that needs more scratch allocates, and a call made while its
- * stream is being captured that would need to allocate takes the static
- * schedule.  A wait gives up after 2 s: the rollout stops, its outputs are
+ * taken.  A launch first waits, on its stream, for the launch that had its
+ * region before, so rollouts of one system may be in flight on any number of
+ * streams (a fifth chunked one starts after the first).  Launches captured into
+ * CUDA graphs take turns over four regions of their own: more than four of one
+ * system in graphs that replay at the same time can zero a region a running
+ * kernel still uses and silently corrupt its results.  A captured launch is
+ * cut only where two chunks of 16 steps fit.  The first call that needs more
+ * scratch allocates, and a call made while its stream is being captured that
+ * would need to allocate takes the static schedule.  A wait gives up after 2 s: the rollout stops, its outputs are
  * incomplete and brax_sync_status reports BRAX_ERR_TIMEOUT. */
 int brax_rollout(const brax_system* sys, int64_t n_envs, int32_t T, int32_t K, const float* state0,
                  const float* actions, float* state_T, float* checkpoints, float* torso_traj,
@@ -281,8 +283,8 @@ int brax_workspace_size(const brax_system* sys, int64_t n_envs, int32_t T, int32
  * device scratch of at least
  * brax_workspace_size bytes, 256-byte aligned.  When the blocks do not fill
  * a whole number of resident waves the launch takes the chunked schedule of
- * brax_rollout over checkpoint segments (last first), with the same scratch
- * ring, allocation and concurrency limit. */
+ * brax_rollout over checkpoint segments (last first), with the same scratch,
+ * allocation and order of concurrent launches. */
 int brax_rollout_backward(const brax_system* sys, int64_t n_envs, int32_t T, int32_t K, const float* state0,
                           const float* actions, const float* checkpoints, const float* g_state_T,
                           const float* g_torso_traj, float* g_actions, float* g_state0, void* workspace,
@@ -326,8 +328,7 @@ int brax_batch_offsets(const brax_batch* batch, int32_t T, int32_t K, int32_t i,
  * concatenated blocks).  It takes the chunked schedule described at
  * brax_rollout when the batch's blocks do not fill a whole number of resident
  * waves (the scratch is the batch's, with the same allocation on first need
- * and the same limit of four chunked launches of the batch in flight; a wait
- * that gives up is reported by the brax_sync_status of the system whose
+ * and the same order of concurrent launches; a wait that gives up is reported by the brax_sync_status of the system whose
  * environments were waited for). */
 int brax_batch_rollout(const brax_batch* batch, int32_t T, int32_t K, const float* state0, const float* actions,
                        float* state_T, float* checkpoints, float* torso_traj, void* stream);

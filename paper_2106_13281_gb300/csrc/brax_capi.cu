@@ -686,6 +686,7 @@ Seg make_seg(const brax_system* s, int groups, int64_t n_envs) {
 // check): a quarter step, or kWideOverhead.
 struct SchedPlan {
   int n_chunks = 0, chunk_steps = 0;
+  bool captured = true;  // also when the launch is captured into a CUDA graph
 };
 // The plan for `slots` resident blocks (host arithmetic only).
 SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t slots, int min_chunk,
@@ -724,16 +725,22 @@ SchedPlan plan_schedule_slots(int mode, int chunk, int64_t units, int T, int64_t
 // The shortest chunk, in steps: short rollouts gain from short chunks too
 // (16,384 bipeds x 50, 3.37 waves: 234 us a step in chunks of 17, 228 of 10).
 constexpr int kMinChunk = 4;
+// A launch captured into a CUDA graph is cut only where two chunks of this many
+// steps fit: the regions of captured launches are few, and no event can say
+// when a replay has left one.
+constexpr int kMinCapturedChunk = 16;
 // A chunk of the wide limb kernel costs about 1.5 steps more than its steps,
 // from 65,536 quadrupeds in chunks of 20 steps (75.2 us a step) and of 50 (72.2).
 constexpr double kWideOverhead = 1.5;
 // per_sm() gives the resident blocks per SM.  It asks the driver (a microsecond
 // or more, of the ten that a one-step call takes), so only a launch that could
 // be cut asks: not a single step, nor a launch of at most one block an SM.
+// steps: of one unit of T (reverse pass: the checkpoint interval).
 template <class PerSm>
-SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, PerSm per_sm,
-                        int min_chunk = kMinChunk, double overhead = 0.25) {
+SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, PerSm per_sm, int steps = 1,
+                        double overhead = 0.25) {
   if (mode == 0 || T < 2 || units < 1) return SchedPlan{};
+  const int min_chunk = (kMinChunk + steps - 1) / steps;
   int n_sm = 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
@@ -742,23 +749,37 @@ SchedPlan plan_schedule(int mode, int chunk, int device, int64_t units, int T, P
   if (mode == 1 && (units <= n_sm || T < 2 * min_chunk)) return SchedPlan{};
   const int blocks = per_sm();
   if (blocks < 1) return SchedPlan{};
-  return plan_schedule_slots(mode, chunk, units, T, (int64_t)blocks * n_sm, min_chunk, overhead);
+  SchedPlan p = plan_schedule_slots(mode, chunk, units, T, (int64_t)blocks * n_sm, min_chunk, overhead);
+  p.captured = mode != 1 || (T + 1) / 2 >= (kMinCapturedChunk + steps - 1) / steps;
+  return p;
 }
 
+// An eager launch's hold on its scheduler region, from taking it until the
+// launch is enqueued: the region's next user waits for the event recorded here.
+struct SchedHold {
+  std::unique_lock<std::mutex> lk;
+  cudaEvent_t done = nullptr;
+  cudaStream_t st = nullptr;
+  ~SchedHold() {
+    if (done) cudaEventRecord(done, st);
+  }
+};
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
+  cudaGetLastError();
+  return true;
+}
 // One region of a scheduler scratch for a launch of `units` units (null when
 // it cannot be had: the caller then runs the static schedule).  Growing the
 // scratch allocates, which a stream under capture does not allow.
-int32_t* sched_region(SchedScratch& sc, int64_t units, cudaStream_t st) {
-  std::lock_guard<std::mutex> lk(sc.mu);
+int32_t* sched_region(SchedScratch& sc, int64_t units, cudaStream_t st, bool capturing, SchedHold& hold) {
+  hold.lk = std::unique_lock<std::mutex>(sc.mu);
   if (units > sc.units) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return nullptr;
-    }
+    if (capturing) return nullptr;
     const int64_t cap = std::max<int64_t>(units, 2 * sc.units);
     int32_t* d = nullptr;
-    if (cudaMalloc(&d, SchedScratch::kRing * (32 + cap) * sizeof(int32_t)) != cudaSuccess) {
+    if (cudaMalloc(&d, 2 * SchedScratch::kRing * (32 + cap) * sizeof(int32_t)) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
@@ -766,13 +787,27 @@ int32_t* sched_region(SchedScratch& sc, int64_t units, cudaStream_t st) {
     sc.d = d;
     sc.units = cap;
   }
-  const int r = sc.next;
-  sc.next = (r + 1) % SchedScratch::kRing;
-  return sc.d + r * (32 + sc.units);
+  const int r = sc.next[capturing];
+  if (!capturing) {
+    cudaEvent_t& done = sc.done[r];
+    if ((!done && cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) ||
+        cudaStreamWaitEvent(st, done, 0) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    hold.done = done;
+    hold.st = st;
+  }
+  sc.next[capturing] = (r + 1) % SchedScratch::kRing;
+  return sc.d + (capturing ? SchedScratch::kRing + r : r) * (32 + sc.units);
 }
 void sched_free(SchedScratch& sc) {
   if (sc.d) cudaFree(sc.d);
   for (int32_t* d : sc.retired) cudaFree(d);
+  for (cudaEvent_t& e : sc.done) {
+    if (e) cudaEventDestroy(e);
+    e = nullptr;
+  }
   sc.d = nullptr;
   sc.retired.clear();
 }
@@ -789,16 +824,20 @@ struct FixedRegion {
 
 // Fill L.sc for a chunked launch of `units` units when the plan asks for one
 // and scratch can be had; returns the grid (one block per item, or `units`).
-// Fails only if zeroing the scratch region fails.
+// Fails only if zeroing the scratch region fails.  `hold` lives until the
+// launch is enqueued.
 cudaError_t apply_schedule(const SchedPlan& pl, SchedScratch& sc, int first_item, int64_t wait_ns, int64_t units,
-                           Launch& L, int64_t* grid, cudaStream_t st, const FixedRegion& fr = FixedRegion{}) {
+                           Launch& L, int64_t* grid, cudaStream_t st, SchedHold& hold,
+                           const FixedRegion& fr = FixedRegion{}) {
   *grid = units;
   if (pl.n_chunks == 0) return cudaSuccess;
   int32_t* region = nullptr;
   if (fr.use) {
     if (fr.fixed && fr.bytes >= (size_t)(32 + units) * sizeof(int32_t)) region = fr.fixed;
   } else {
-    region = sched_region(sc, units, st);
+    const bool capturing = is_capturing(st);
+    if (capturing && !pl.captured) return cudaSuccess;
+    region = sched_region(sc, units, st, capturing, hold);
   }
   if (!region) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(region, 0, (32 + units) * sizeof(int32_t), st);
@@ -1095,12 +1134,13 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     sg.ccount = contact_count;
     apply_env(s, sg, env);
     L.seg[0] = sg;
-    const SchedPlan pl =
-        plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T, [&] { return limb_blocks_per_sm(ll); }, kMinChunk,
-                      ll.split ? 0.25 : kWideOverhead);
+    SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
+                                 [&] { return limb_blocks_per_sm(ll); }, 1, ll.split ? 0.25 : kWideOverhead);
+    if (ll.split && s->sched_mode == 1) pl.captured = false;
     int64_t launch_grid;
+    SchedHold hold;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
-                                   as_stream(stream), fr);
+                                   as_stream(stream), hold, fr);
     s->last_grid = launch_grid;
     s->last_chunks = L.sc.n_chunks;
     s->last_chunk_steps = L.sc.chunk_steps;
@@ -1142,8 +1182,9 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
                                        [&] { return pair_blocks_per_sm(pvariant, threads, smem); });
     int64_t launch_grid;
+    SchedHold hold;
     cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
-                                   as_stream(stream), fr);
+                                   as_stream(stream), hold, fr);
     s->last_grid = launch_grid;
     s->last_chunks = L.sc.n_chunks;
     s->last_chunk_steps = L.sc.chunk_steps;
@@ -1173,8 +1214,9 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
                                      [&] { return rollout_blocks_per_sm(s->variant, s->general, shared, threads, smem); });
   int64_t launch_grid;
+  SchedHold hold;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
-                                 as_stream(stream), fr);
+                                 as_stream(stream), hold, fr);
   s->last_grid = launch_grid;
   s->last_chunks = L.sc.n_chunks;
   s->last_chunk_steps = L.sc.chunk_steps;
@@ -1496,7 +1538,8 @@ extern "C" int brax_batch_rollout(const brax_batch* b, int32_t T, int32_t K, con
   const SchedPlan pl = plan_schedule(b->sched_mode, b->sched_chunk, device, grid, T,
                                      [&] { return rollout_blocks_per_sm(variant, general, shared, threads, smem); });
   int64_t launch_grid;
-  cudaError_t e = apply_schedule(pl, b->sched, 0, 2000000000LL, grid, L, &launch_grid, as_stream(stream));
+  SchedHold hold;
+  cudaError_t e = apply_schedule(pl, b->sched, 0, 2000000000LL, grid, L, &launch_grid, as_stream(stream), hold);
   if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, shared, as_stream(stream));
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout");
 }
@@ -1644,9 +1687,10 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
                                      [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, false, threads, smem); },
-                                     (kMinChunk + K - 1) / K);
+                                     K);
   int64_t launch_grid;
-  cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, fr);
+  SchedHold hold;
+  cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, hold, fr);
   if (e == cudaSuccess)
     e = launch_rollout_backward(L, (int)launch_grid, threads, smem, variant, s->general, s->iso, shared, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout_backward");
@@ -1787,9 +1831,10 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   const size_t smem = shared ? pl.smem_with : pl.smem;
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
                                      [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.keep, pl.threads, smem); },
-                                     (kMinChunk + K - 1) / K);
+                                     K);
   int64_t launch_grid;
-  cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st);
+  SchedHold hold;
+  cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st, hold);
   if (e == cudaSuccess)
     e = launch_rollout_backward(L, (int)launch_grid, pl.threads, smem, variant, pl.general, pl.iso, shared, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout_backward");

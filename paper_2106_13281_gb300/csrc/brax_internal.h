@@ -15,15 +15,18 @@ namespace brax {
 // environments, the wide one (two environments a lane), the split one (one
 // limb body a lane).
 constexpr int kLimbVariant = 5, kLimbWide = 6, kLimbSplit = 7;
-// Scheduler scratch of chunked rollouts: kRing regions of (32 + units) int32,
-// taken in turn by successive launches so that rollouts on different streams
-// do not share one; replaced buffers are freed with the owner.
+// Scheduler scratch of chunked rollouts: regions of (32 + units) int32, kRing
+// for eager launches, taken in turn, and kRing for launches captured into CUDA
+// graphs.  An eager launch first waits, on its stream, for the launch that had
+// its region before (done[r]), so any number of them may be in flight on any
+// streams.  Replaced buffers are freed with the owner.
 struct SchedScratch {
   static constexpr int kRing = 4;
   std::mutex mu;
   int32_t* d = nullptr;
   int64_t units = 0;
-  int next = 0;
+  int next[2] = {0, 0};             // eager, captured
+  cudaEvent_t done[kRing] = {};     // the end of the last eager launch in a region
   std::vector<int32_t*> retired;
 };
 }  // namespace brax

@@ -893,7 +893,7 @@ int brax_system_create(const brax_desc* desc, brax_system** out) {
       cudaFree(s->d_blob);
       cudaFree(s->d_status);
       delete s;
-      return fail(BRAX_ERR_OUT_OF_MEMORY, "brax_system_create: the constant parameter pool (60 KB per device) is full");
+      return fail(BRAX_ERR_OUT_OF_MEMORY, "brax_system_create: the constant parameter pool (64 KB per device) is full");
     }
     if (off < -1) e = (cudaError_t)(-2 - off);
     else s->pool_off = off;

@@ -13,7 +13,7 @@ namespace brax {
 // Constant-memory pool holding the parameter blobs of all live systems.  A
 // warp reads its body's parameters with a warp-uniform index, so the loads go
 // through the constant cache and the uniform datapath, not the LSU.
-constexpr int kPoolBytes = 61440;
+constexpr int kPoolBytes = 65280;  // of the 64 KB a module's constants may take
 
 // One system's share of a launch.  A thread block runs G groups of 32
 // environments of one system; group g's warps are bodies 0..B-1 (warp =

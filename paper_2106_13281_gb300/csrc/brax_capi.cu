@@ -27,6 +27,7 @@ int fail(int code, const std::string& msg) {
   return code;
 }
 int cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: the next call does not meet it again
   return fail(BRAX_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 

@@ -76,3 +76,18 @@ def test_large_blocks_fit_and_match_solo(name):
         assert close(gs[so:so + rs.numel()], rs, rs.abs().max().item() + 1.0)
         assert close(ga[ao:ao + ra.numel()], ra, ra.abs().max().item() + 1.0)
         s.sync_status()
+
+
+def test_a_refused_launch_leaves_no_error_behind():
+    """The reverse pass of 28 bodies needs more shared memory than a block has
+    and is refused with an error code; the next call runs."""
+    from paper_2106_13281_gb300.binding import BraxError
+    from paper_2106_13281_gb300.system import BraxSystem
+    s = BraxSystem(chain(28))
+    st = s.default_qp(32)
+    a = torch.zeros((1, 32, s.A), device="cuda")
+    ck = s.rollout(st, a, K=1, checkpoints=True)["checkpoints"]
+    with pytest.raises(BraxError):
+        s.rollout_backward(st, a, ck, torch.ones_like(st), K=1)
+    assert torch.equal(s.default_qp(32), st)
+    s.sync_status()

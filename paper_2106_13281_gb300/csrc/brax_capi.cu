@@ -1071,19 +1071,33 @@ void apply_env(const brax_system* s, Seg& sg, const EnvOut* env) {
 //   2 limbs  5.5/14.5/13.4   9.3/14.5/13.5  13.7/14.5/16.8  17.6/14.6/16.8  19.8/24.7/22.0  23.9/24.7/22.1  35.5/26.5/28.2
 //   4 limbs  5.5/13.4/18.2   9.3/13.4/18.3  13.8/13.5/18.5  17.8/13.6/18.9  20.0/22.9/26.3  24.1/23.1/26.5  35.9/24.5/30.5
 //   8 limbs  5.8/13.3/28.0   9.7/13.3/29.1  14.5/13.4/29.7  18.6/13.4/31.8  21.0/22.7/35.8  25.4/22.7/40.8  37.8/24.3/52.8
-int limb_kind(const brax_system* s, int64_t n_envs, int n_sm) {
-  if (s->n_limbs == 0 || s->pair_variant < kLimbVariant) return 0;
-  if (s->pair_variant != kLimbVariant) return s->pair_variant;
-  const int64_t per_warp = limb_warp_envs(s->n_limbs, true), split_warps = (n_envs + per_warp - 1) / per_warp;
+// With one limb the wide kernel's lead is small, so what it costs to start (its
+// table, 250 registers a thread) and what the environment layer costs it decide
+// between 8 and 16 warps (us a launch, wide / body layout; 14 warps: 1 step
+// 31.2/29.1, 20 steps 265/299, 20 steps with the environment layer 348/334; 10
+// warps: 27.3/24.8, 261/265, 345/292).  A launch of one step is not cut into
+// chunks and pays the wide kernel's last step of 16 warps in full: with one or
+// two limbs the body layout wins in the first half of it (33 warps, 2 limbs:
+// 54.2/50.4; 45 warps: 57.5/59.9).
+int limb_rule(int n_limbs, int64_t n_envs, int T, bool env, int n_sm) {
+  const int64_t per_warp = limb_warp_envs(n_limbs, true), split_warps = (n_envs + per_warp - 1) / per_warp;
   auto up_to = [&](int warps) { return split_warps <= (int64_t)warps * n_sm; };
-  if (s->n_limbs == 1) {
+  if (n_limbs == 1) {
     if (up_to(4)) return kLimbSplit;
-    return up_to(8) || (!up_to(16) && up_to(22)) ? 0 : kLimbWide;
+    if (up_to(16)) return !up_to(8) && !env && T >= (up_to(12) ? 16 : 4) ? kLimbWide : 0;
+    if (up_to(22)) return 0;
+  } else {
+    if (up_to(n_limbs == 2 ? 12 : 8)) return kLimbSplit;
+    if (up_to(16)) return kLimbWide;
+    if (up_to(20)) return kLimbSplit;
+    if (n_limbs == 2 && up_to(25)) return 0;
   }
-  if (up_to(s->n_limbs == 2 ? 12 : 8)) return kLimbSplit;
-  if (up_to(16)) return kLimbWide;
-  if (up_to(20)) return kLimbSplit;
-  return s->n_limbs == 2 && up_to(25) ? 0 : kLimbWide;
+  const bool first_half = (split_warps - 1) % (16LL * n_sm) < 8LL * n_sm;
+  return n_limbs <= 2 && T == 1 && first_half ? 0 : kLimbWide;
+}
+int limb_kind(const brax_system* s, int64_t n_envs, int T, bool env, int n_sm) {
+  if (s->n_limbs == 0 || s->pair_variant < kLimbVariant) return 0;
+  return s->pair_variant == kLimbVariant ? limb_rule(s->n_limbs, n_envs, T, env, n_sm) : s->pair_variant;
 }
 
 int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, const float* state0,
@@ -1109,7 +1123,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
     cudaGetLastError();
     n_sm = 1;
   }
-  const int kind = s->pair_mode == 1 ? limb_kind(s, n_envs, n_sm) : 0;
+  const int kind = s->pair_mode == 1 ? limb_kind(s, n_envs, T, env != nullptr, n_sm) : 0;
   if (kind != 0) {
     LimbLaunch ll;
     ll.n_limbs = s->n_limbs;
@@ -1228,6 +1242,10 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
 }  // namespace
 
 extern "C" {
+
+int brax_internal_limb_rule(int32_t n_limbs, int64_t n_envs, int32_t T, int32_t env, int32_t n_sm) {
+  return limb_rule(n_limbs, n_envs, T, env != 0, n_sm);
+}
 
 int brax_rollout(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, const float* state0,
                  const float* actions, float* state_T, float* checkpoints, float* torso_traj, int32_t* contact_count,

@@ -88,6 +88,9 @@ extern "C" int brax_batch_set_schedule(brax_batch* b, int32_t mode, int32_t chun
 // only, for tests): n_chunks = 0 means the static schedule.
 extern "C" int brax_internal_plan_schedule(int32_t mode, int32_t chunk_steps, int64_t units, int32_t T, int64_t slots,
                                            int32_t min_chunk, int32_t* n_chunks, int32_t* steps);
+// The kernel the limb layout's rule picks (host arithmetic only, for tests):
+// kLimbSplit, kLimbWide or 0 for the body layout.
+extern "C" int brax_internal_limb_rule(int32_t n_limbs, int64_t n_envs, int32_t T, int32_t env, int32_t n_sm);
 // The launch of the system's last brax_rollout: blocks launched, chunks of
 // the chunked schedule (0 = static schedule) and steps per chunk.
 extern "C" int brax_system_last_rollout(const brax_system* s, int64_t* grid, int32_t* n_chunks, int32_t* chunk_steps);

@@ -472,7 +472,7 @@ __device__ __forceinline__ void bwd_substep_iso(const SysP& S, const PlaneP* pla
 // each: 0.387 -> 0.326.  The general kernel takes either; the hinge-only ones
 // are built for each (kKeep), since the choice at run time cost the other
 // layout 1.5 % (65,536 quadrupeds, K = 1).
-template <bool kGeneral, bool kIso, bool kShared, bool kKeep>
+template <bool kGeneral, bool kIso, int kParams, bool kKeep>
 __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -502,13 +502,14 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
   const Seg& sg = L.seg[si];
   const unsigned char* blob = c_pool + sg.pool_off;
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
-  if constexpr (kShared) {  // as in the forward kernel
-    blob = smem + sg.groups * bwd_group_floats(sg.B, sg.P) * sizeof(float) - sizeof(SysP);
-    copy_params(sg.blob, smem + sg.groups * bwd_group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P, S.n_planes);
+  unsigned char* const params = smem + sg.groups * bwd_group_floats(sg.B, sg.P) * sizeof(float);
+  if constexpr (kParams != kInPool) {  // as in the forward kernel
+    copy_params<kParams>(sg.blob, params, sg.B, sg.P, S.n_planes);
     group_sync(0, blockDim.x);
   }
+  if constexpr (kParams == kAllShared) blob = params - sizeof(SysP);
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
-  const PairP* pairs = reinterpret_cast<const PairP*>(blob + blob_pairs_off(sg.B));
+  const PairP* pairs = reinterpret_cast<const PairP*>(kParams == kPairsShared ? params : blob + blob_pairs_off(sg.B));
   const PlaneP* planes = reinterpret_cast<const PlaneP*>(blob + blob_planes_off(sg.B, sg.P));
   const int B = sg.B, P = sg.P;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -684,36 +685,38 @@ __device__ __forceinline__ void rollout_bwd_body(const Launch& L) {
 // groups per SM), which holds more of the adjoint's live values than the
 // 96 registers (576, 1) gives.  Each is compiled for three kinds of system:
 // hinge-only, hinge-only with isotropic inertia (bwd_substep_iso), general.
-template <int MAXT, int MINB, bool kGeneral, bool kIso, bool kShared, bool kKeep>
+template <int MAXT, int MINB, bool kGeneral, bool kIso, int kParams, bool kKeep>
 __global__ void __launch_bounds__(MAXT, MINB) rollout_bwd_kernel(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso, kShared, kKeep>(L);
+  rollout_bwd_body<kGeneral, kIso, kParams, kKeep>(L);
 }
-template <bool kGeneral, bool kIso, bool kShared, bool kKeep>
+template <bool kGeneral, bool kIso, int kParams, bool kKeep>
 __global__ void __maxnreg__(112) rollout_bwd_kernel_r112(const __grid_constant__ Launch L) {
-  rollout_bwd_body<kGeneral, kIso, kShared, kKeep>(L);
+  rollout_bwd_body<kGeneral, kIso, kParams, kKeep>(L);
 }
 
 using BwdKernel = void (*)(const Launch);
-template <bool G, bool I, bool Sh, bool Kp>
+template <bool G, bool I, int Pr, bool Kp>
 static BwdKernel bwd_kernel_t(int variant) {
   switch (variant) {
-    case 0: return rollout_bwd_kernel<384, 2, G, I, Sh, Kp>;
-    case 1: return rollout_bwd_kernel<576, 1, G, I, Sh, Kp>;
-    case 3: return rollout_bwd_kernel<288, 3, G, I, Sh, Kp>;
-    case 4: return rollout_bwd_kernel_r112<G, I, Sh, Kp>;
-    default: return rollout_bwd_kernel<1024, 1, G, I, Sh, Kp>;
+    case 0: return rollout_bwd_kernel<384, 2, G, I, Pr, Kp>;
+    case 1: return rollout_bwd_kernel<576, 1, G, I, Pr, Kp>;
+    case 3: return rollout_bwd_kernel<288, 3, G, I, Pr, Kp>;
+    case 4: return rollout_bwd_kernel_r112<G, I, Pr, Kp>;
+    default: return rollout_bwd_kernel<1024, 1, G, I, Pr, Kp>;
   }
 }
-static BwdKernel bwd_kernel(int variant, bool general, bool iso, bool shared, bool keep) {
+static BwdKernel bwd_kernel(int variant, bool general, bool iso, int params, bool keep) {
+  if (general && params == kPairsShared) return rollout_bwd_kernel<576, 1, true, false, kPairsShared, false>;
   if (general)
-    return shared ? bwd_kernel_t<true, false, true, false>(variant) : bwd_kernel_t<true, false, false, false>(variant);
+    return params == kAllShared ? bwd_kernel_t<true, false, kAllShared, false>(variant)
+                                : bwd_kernel_t<true, false, kInPool, false>(variant);
   if (keep)
-    return iso ? bwd_kernel_t<false, true, false, true>(variant) : bwd_kernel_t<false, false, false, true>(variant);
-  return iso ? bwd_kernel_t<false, true, false, false>(variant) : bwd_kernel_t<false, false, false, false>(variant);
+    return iso ? bwd_kernel_t<false, true, kInPool, true>(variant) : bwd_kernel_t<false, false, kInPool, true>(variant);
+  return iso ? bwd_kernel_t<false, true, kInPool, false>(variant) : bwd_kernel_t<false, false, kInPool, false>(variant);
 }
 
-int backward_blocks_per_sm(int variant, bool general, bool iso, bool shared, bool keep, int threads, size_t smem) {
-  const BwdKernel k = bwd_kernel(variant, general, iso, shared, keep);
+int backward_blocks_per_sm(int variant, bool general, bool iso, int params, bool keep, int threads, size_t smem) {
+  const BwdKernel k = bwd_kernel(variant, general, iso, params, keep);
   if (allow_smem(k, smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
@@ -726,8 +729,8 @@ int backward_variant_max_threads(int variant) {
 }
 
 cudaError_t launch_rollout_backward(const Launch& L, int grid, int threads, size_t smem, int variant, bool general,
-                                    bool iso, bool shared, cudaStream_t st) {
-  const BwdKernel k = bwd_kernel(variant, general, iso, shared, L.keep != 0);
+                                    bool iso, int params, cudaStream_t st) {
+  const BwdKernel k = bwd_kernel(variant, general, iso, params, L.keep != 0);
   cudaError_t e = allow_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<grid, threads, smem, st>>>(L);

@@ -569,12 +569,11 @@ std::vector<unsigned char> build_blob(const brax_desc& d, int* n_planes_out, int
 
 namespace {
 
-// Bytes of a system's parameters when a general kernel keeps them in shared memory.
+// Bytes of a system's parameters when a general kernel keeps the pairs', or all
+// of them, in shared memory.
+size_t pair_smem(const brax_system* s) { return (size_t)s->P * sizeof(PairP); }
 size_t param_smem(const brax_system* s) { return (size_t)params_bytes(s->B, s->P, s->n_planes); }
-// Whether a general launch of `with` bytes of shared memory (groups and
-// parameters) fits a block.  The parameters then come from shared memory: the
-// biped's substep takes 6.7 us there and 10.8 from the constant cache (4,864
-// environments, one group an SM).
+// Whether a launch of `with` bytes of shared memory fits a block.
 bool fits_block(size_t with, int device) {
   int optin = 0;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
@@ -582,6 +581,50 @@ bool fits_block(size_t with, int device) {
     return false;
   }
   return with + 64 <= (size_t)optin;
+}
+
+// Where a general launch of `units` blocks reads its parameters (ParamsIn).  smem:
+// a block's bytes of shared memory with the parameters in the pool, with the
+// pairs' and with all parameters behind the groups.
+//
+// Shared memory serves what the constant cache misses: the biped's substep takes
+// 6.7 us with all parameters there and 10.8 from the pool (4,864 environments,
+// one group an SM).  But an SM's shared memory is cut from its L1 cache in steps
+// (carve-outs), and the kernels spill registers (190 to 340 bytes a thread) to
+// L1: a launch whose bodies' parameters take the SM a step further pays more for
+// its spills than it gains.  Us for 10 steps, pairs / all shared: 9 bodies and 10
+// pairs, 14,592 environments 413/463; 7 bodies and 9 pairs 368/428; 9 bodies
+// without pairs, 65,536 environments 1,542/1,589, but 1,000 (one block an SM)
+// 196/185.  At the same step all is as good or better: 9 bodies and 19 pairs,
+// 1,000 environments 285/270; 7 bodies and 15 pairs (four blocks an SM with the
+// pairs', three with all) 458/410.  And half the blocks an SM is too few once
+// there are more blocks than SMs: 12 bodies and 45 pairs, 14,592 environments
+// 1,042/1,392, 1,000 environments 488/471.
+// The reverse kernel spills more and reads more parameters; once two blocks share
+// an SM their spills leave L1 either way.  4 steps: 9 bodies without pairs, 100
+// environments 412/457, 40,000 2,881/2,732; 5 bodies and one pair (four blocks an
+// SM) 300/389, 1,446/1,522.  (Its pairs-only kernel is compiled for the default
+// launch, variant 1.)
+int place_params(bool reverse, int variant, int threads, const size_t smem[3], int64_t units, int device) {
+  if (!fits_block(smem[kAllShared], device)) return kInPool;
+  if (reverse && variant != 1) return kAllShared;
+  int n_sm = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) cudaGetLastError();
+  // registers a thread by variant: 80, 96, 64, 72, 112
+  static const int kWarps[5] = {25, 21, 32, 28, 18};
+  static const size_t kCarve[] = {8, 16, 32, 64, 100, 132, 164, 196, 228};
+  auto blocks = [&](int in) {
+    return std::max<size_t>(1, std::min<size_t>(32 * kWarps[variant] / threads, (228 << 10) / (smem[in] + 1024)));
+  };
+  auto step = [&](int in) {
+    const size_t kb = (blocks(in) * (smem[in] + 1024) + 1023) >> 10;
+    return std::lower_bound(std::begin(kCarve), std::end(kCarve), kb) - std::begin(kCarve);
+  };
+  const bool one_an_sm = units <= n_sm, pairs = smem[kPairsShared] > smem[kInPool];
+  bool all = one_an_sm || 2 * blocks(kAllShared) > blocks(kPairsShared);
+  if (step(kAllShared) > step(kPairsShared))
+    all = all && (reverse ? !one_an_sm && blocks(kAllShared) < 3 : one_an_sm && !pairs);
+  return all ? kAllShared : pairs ? kPairsShared : kInPool;
 }
 
 size_t group_bytes(const brax_system* s) { return (size_t)group_floats(s->B, s->P) * sizeof(float); }
@@ -1222,12 +1265,14 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   sg.ccount = contact_count;
   apply_env(s, sg, env);
   L.seg[0] = sg;
-  size_t smem = s->groups * group_bytes(s);
-  const bool shared = s->general && fits_block(smem + param_smem(s), s->device);
-  if (shared) smem += param_smem(s);
   const int threads = 32 * s->B * s->groups;
+  const size_t base = s->groups * group_bytes(s), sizes[3] = {base, base + pair_smem(s), base + param_smem(s)};
+  // (the environment layer's kernels have launch bounds of their own)
+  const int bounds = !env ? s->variant : threads <= 576 ? 1 : 2;
+  const int params = s->general ? place_params(false, bounds, threads, sizes, grid, s->device) : kInPool;
+  const size_t smem = sizes[params];
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, T,
-                                     [&] { return rollout_blocks_per_sm(s->variant, s->general, shared, threads, smem); });
+                                     [&] { return rollout_blocks_per_sm(s->variant, s->general, params, threads, smem); });
   int64_t launch_grid;
   SchedHold hold;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid,
@@ -1235,7 +1280,7 @@ int rollout_impl(const brax_system* s, int64_t n_envs, int32_t T, int32_t K, con
   s->last_grid = launch_grid;
   s->last_chunks = L.sc.n_chunks;
   s->last_chunk_steps = L.sc.chunk_steps;
-  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, s->variant, s->general, shared, as_stream(stream));
+  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, s->variant, s->general, params, as_stream(stream));
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout");
 }
 
@@ -1495,15 +1540,15 @@ int brax_batch_offsets(const brax_batch* b, int32_t T, int32_t K, int32_t i, int
 
 namespace brax_batch_impl {
 // Fill a launch table for the batch; pointers offset per system.
-int make_launch(const brax_batch* b, int32_t T, int32_t K, Launch& L, int* grid, int* threads, size_t* smem,
-                size_t* smem_with, bool* general) {
+int make_launch(const brax_batch* b, int32_t T, int32_t K, Launch& L, int* grid, int* threads, size_t smem[3],
+                bool* general) {
   *general = false;
   std::memset(&L, 0, sizeof(L));
   L.n_segs = (int)b->sys.size();
   L.T = T;
   L.K = K;
   int cta = 0;
-  size_t sm = 0, sw = 0;  // shared memory without and with the parameters
+  smem[kInPool] = smem[kPairsShared] = smem[kAllShared] = 0;
   const std::vector<int> order = batch_order(b);
   for (int j = 0; j < L.n_segs; ++j) {
     const int i = order[j];
@@ -1514,15 +1559,15 @@ int make_launch(const brax_batch* b, int32_t T, int32_t K, Launch& L, int* grid,
     sg.cta_begin = cta;
     sg.cta_end = cta + (int)nb;
     cta += (int)nb;
-    sm = std::max(sm, (size_t)G * group_bytes(s));
-    sw = std::max(sw, (size_t)G * group_bytes(s) + param_smem(s));
+    const size_t base = G * group_bytes(s);
+    smem[kInPool] = std::max(smem[kInPool], base);
+    smem[kPairsShared] = std::max(smem[kPairsShared], base + pair_smem(s));
+    smem[kAllShared] = std::max(smem[kAllShared], base + param_smem(s));
     *general = *general || s->general;
     L.seg[j] = sg;
   }
   *grid = cta;
   *threads = 32 * b->warps;
-  *smem = sm;
-  *smem_with = sw;
   return BRAX_OK;
 }
 }  // namespace brax_batch_impl
@@ -1534,9 +1579,9 @@ extern "C" int brax_batch_rollout(const brax_batch* b, int32_t T, int32_t K, con
   if (K < 1) K = 1;
   Launch L;
   int grid, threads;
-  size_t smem, smem_with;
+  size_t sizes[3];
   bool general;
-  brax_batch_impl::make_launch(b, T, K, L, &grid, &threads, &smem, &smem_with, &general);
+  brax_batch_impl::make_launch(b, T, K, L, &grid, &threads, sizes, &general);
   const std::vector<int> order = batch_order(b);
   for (int j = 0; j < L.n_segs; ++j) {
     int64_t so, ao, to, co;
@@ -1552,14 +1597,14 @@ extern "C" int brax_batch_rollout(const brax_batch* b, int32_t T, int32_t K, con
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_batch_rollout: block too large");
   int device = 0;
   cudaGetDevice(&device);
-  const bool shared = general && fits_block(smem_with, device);
-  if (shared) smem = smem_with;
+  const int params = general ? place_params(false, variant, threads, sizes, grid, device) : kInPool;
+  const size_t smem = sizes[params];
   const SchedPlan pl = plan_schedule(b->sched_mode, b->sched_chunk, device, grid, T,
-                                     [&] { return rollout_blocks_per_sm(variant, general, shared, threads, smem); });
+                                     [&] { return rollout_blocks_per_sm(variant, general, params, threads, smem); });
   int64_t launch_grid;
   SchedHold hold;
   cudaError_t e = apply_schedule(pl, b->sched, 0, 2000000000LL, grid, L, &launch_grid, as_stream(stream), hold);
-  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, shared, as_stream(stream));
+  if (e == cudaSuccess) e = launch_rollout(L, (int)launch_grid, threads, smem, variant, general, params, as_stream(stream));
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout");
 }
 
@@ -1700,18 +1745,18 @@ int rollout_backward_impl(const brax_system* s, int64_t n_envs, int32_t T, int32
       (s->bwd_variant >= 0 && threads <= backward_variant_max_threads(s->bwd_variant)) ? s->bwd_variant
                                                                                         : pick_bwd_variant(threads);
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_rollout_backward: system too large for one block");
-  size_t smem = backward_smem_bytes(s->B, s->P, 1);
-  const bool shared = s->general && fits_block(smem + param_smem(s), s->device);
-  if (shared) smem += param_smem(s);
+  const size_t base = backward_smem_bytes(s->B, s->P, 1), sizes[3] = {base, base + pair_smem(s), base + param_smem(s)};
+  const int params = s->general ? place_params(true, variant, threads, sizes, grid, s->device) : kInPool;
+  const size_t smem = sizes[params];
   const int nseg = (T + K - 1) / K;
   const SchedPlan pl = plan_schedule(s->sched_mode, s->sched_chunk, s->device, grid, nseg,
-                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, shared, false, threads, smem); },
+                                     [&] { return backward_blocks_per_sm(variant, s->general, s->iso, params, false, threads, smem); },
                                      K);
   int64_t launch_grid;
   SchedHold hold;
   cudaError_t e = apply_schedule(pl, s->sched, s->sched_first, s->sched_wait_ns, grid, L, &launch_grid, st, hold, fr);
   if (e == cudaSuccess)
-    e = launch_rollout_backward(L, (int)launch_grid, threads, smem, variant, s->general, s->iso, shared, st);
+    e = launch_rollout_backward(L, (int)launch_grid, threads, smem, variant, s->general, s->iso, params, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_rollout_backward");
 }
 }  // namespace
@@ -1743,7 +1788,7 @@ namespace {
 // groups of 32 environments, its workspace block starts at ws_off[i].
 struct BwdBatchPlan {
   int grid = 0, threads = 0;
-  size_t smem = 0, smem_with = 0, ws_bytes = 0;  // smem_with: with the parameters in shared memory
+  size_t smem[3] = {0, 0, 0}, ws_bytes = 0;  // smem: by where the parameters are (ParamsIn)
   bool general = false, iso = true;
   std::vector<int> groups, blocks;  // by system
   std::vector<int> order;           // the systems as their blocks start
@@ -1773,8 +1818,10 @@ BwdBatchPlan plan_batch_layout(const brax_batch* b, int32_t K, bool keep) {
                       (size_t)backward_ws_floats_per_group(s->B, s->P, keep ? 0 : K, keep ? K * S->substeps : S->substeps) *
                       sizeof(float);
     pl.ws_bytes += (wb + 255) & ~size_t(255);
-    pl.smem = std::max(pl.smem, backward_smem_bytes(s->B, s->P, G));
-    pl.smem_with = std::max(pl.smem_with, backward_smem_bytes(s->B, s->P, G) + param_smem(s));
+    const size_t base = backward_smem_bytes(s->B, s->P, G);
+    pl.smem[kInPool] = std::max(pl.smem[kInPool], base);
+    pl.smem[kPairsShared] = std::max(pl.smem[kPairsShared], base + pair_smem(s));
+    pl.smem[kAllShared] = std::max(pl.smem[kAllShared], base + param_smem(s));
     pl.general = pl.general || s->general;
     pl.iso = pl.iso && s->iso;
   }
@@ -1846,16 +1893,16 @@ extern "C" int brax_batch_rollout_backward(const brax_batch* b, int32_t T, int32
   if (variant < 0) return fail(BRAX_ERR_INVALID_ARGUMENT, "brax_batch_rollout_backward: block too large");
   int device = 0;
   cudaGetDevice(&device);
-  const bool shared = pl.general && fits_block(pl.smem_with, device);
-  const size_t smem = shared ? pl.smem_with : pl.smem;
+  const int params = pl.general ? place_params(true, variant, pl.threads, pl.smem, pl.grid, device) : kInPool;
+  const size_t smem = pl.smem[params];
   const SchedPlan sp = plan_schedule(b->sched_mode, b->sched_chunk, device, pl.grid, (T + K - 1) / K,
-                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, shared, pl.keep, pl.threads, smem); },
+                                     [&] { return backward_blocks_per_sm(variant, pl.general, pl.iso, params, pl.keep, pl.threads, smem); },
                                      K);
   int64_t launch_grid;
   SchedHold hold;
   cudaError_t e = apply_schedule(sp, b->sched, 0, 2000000000LL, pl.grid, L, &launch_grid, st, hold);
   if (e == cudaSuccess)
-    e = launch_rollout_backward(L, (int)launch_grid, pl.threads, smem, variant, pl.general, pl.iso, shared, st);
+    e = launch_rollout_backward(L, (int)launch_grid, pl.threads, smem, variant, pl.general, pl.iso, params, st);
   return e == cudaSuccess ? BRAX_OK : cuda_fail(e, "brax_batch_rollout_backward");
 }
 

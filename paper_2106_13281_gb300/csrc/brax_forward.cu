@@ -87,11 +87,12 @@ __device__ __forceinline__ int substep_forward(const SysP& S, const BodyP* bodie
 // unit blockIdx.x for the whole rollout, or, under a chunked schedule
 // (Sched), one chunk of the unit of the item it takes.
 //
-// kShared (general systems): the bodies', pairs' and planes' parameters are
-// read from a copy in shared memory.  A general system's warps read about 28 KB
-// of them a substep, each its own body's and pairs', far more than the constant
-// cache holds (measured on the biped: 20-29 % of its requests miss).
-template <int MAXT, int MINB, bool kGeneral, bool kEnv, bool kShared>
+// kParams (general systems, ParamsIn): the pairs', or the bodies', pairs' and
+// planes' parameters are read from a copy in shared memory.  A general system's
+// warps read up to 28 KB of them a substep, each its own body's and pairs', far
+// more than the constant cache holds (measured on the biped: 20-29 % of its
+// requests miss).
+template <int MAXT, int MINB, bool kGeneral, bool kEnv, int kParams>
 __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_constant__ Launch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
@@ -123,13 +124,14 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
   const Seg& sg = L.seg[si];
   const unsigned char* blob = c_pool + sg.pool_off;
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
-  if constexpr (kShared) {
-    blob = smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float) - sizeof(SysP);
-    copy_params(sg.blob, smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P, S.n_planes);
+  unsigned char* const params = smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float);
+  if constexpr (kParams != kInPool) {
+    copy_params<kParams>(sg.blob, params, sg.B, sg.P, S.n_planes);
     group_sync(0, blockDim.x);
   }
+  if constexpr (kParams == kAllShared) blob = params - sizeof(SysP);
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
-  const PairP* pairs = reinterpret_cast<const PairP*>(blob + blob_pairs_off(sg.B));
+  const PairP* pairs = reinterpret_cast<const PairP*>(kParams == kPairsShared ? params : blob + blob_pairs_off(sg.B));
   const PlaneP* planes = reinterpret_cast<const PlaneP*>(blob + blob_planes_off(sg.B, sg.P));
   const int B = sg.B;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -623,29 +625,31 @@ static int occupancy_k(KernelT k, int threads, size_t smem) {
 // A rollout with the environment layer (Seg::obs) runs the kernels compiled
 // with it, in the (576, 1) launch, or (1024, 1) for larger blocks; the
 // others are compiled without it, so plain rollouts carry none of its code.
-// shared: a general system's parameters in shared memory (smem includes them).
+// params: where a general system's parameters are (smem includes them).
 using RolloutKernel = void (*)(const Launch);
-template <bool G, bool Sh>
+template <bool G, int Pr>
 static RolloutKernel rollout_kernel_t(int variant, int threads, bool env) {
-  if (env) return threads <= 576 ? rollout_kernel<576, 1, G, true, Sh> : rollout_kernel<1024, 1, G, true, Sh>;
+  if (env) return threads <= 576 ? rollout_kernel<576, 1, G, true, Pr> : rollout_kernel<1024, 1, G, true, Pr>;
   switch (variant) {
-    case 0: return rollout_kernel<384, 2, G, false, Sh>;
-    case 1: return rollout_kernel<576, 1, G, false, Sh>;
-    case 3: return rollout_kernel<288, 3, G, false, Sh>;
-    default: return rollout_kernel<1024, 1, G, false, Sh>;
+    case 0: return rollout_kernel<384, 2, G, false, Pr>;
+    case 1: return rollout_kernel<576, 1, G, false, Pr>;
+    case 3: return rollout_kernel<288, 3, G, false, Pr>;
+    default: return rollout_kernel<1024, 1, G, false, Pr>;
   }
 }
-static RolloutKernel rollout_kernel_of(int variant, bool general, bool shared, int threads, bool env) {
-  if (!general) return rollout_kernel_t<false, false>(variant, threads, env);
-  return shared ? rollout_kernel_t<true, true>(variant, threads, env) : rollout_kernel_t<true, false>(variant, threads, env);
+static RolloutKernel rollout_kernel_of(int variant, bool general, int params, int threads, bool env) {
+  if (!general) return rollout_kernel_t<false, kInPool>(variant, threads, env);
+  return params == kAllShared     ? rollout_kernel_t<true, kAllShared>(variant, threads, env)
+         : params == kPairsShared ? rollout_kernel_t<true, kPairsShared>(variant, threads, env)
+                                  : rollout_kernel_t<true, kInPool>(variant, threads, env);
 }
-cudaError_t launch_rollout(const Launch& L, int grid, int threads, size_t smem, int variant, bool general, bool shared,
+cudaError_t launch_rollout(const Launch& L, int grid, int threads, size_t smem, int variant, bool general, int params,
                            cudaStream_t st) {
-  return launch_k(rollout_kernel_of(variant, general, shared, threads, L.seg[0].obs != nullptr), L, grid, threads, smem,
+  return launch_k(rollout_kernel_of(variant, general, params, threads, L.seg[0].obs != nullptr), L, grid, threads, smem,
                   st);
 }
-int rollout_blocks_per_sm(int variant, bool general, bool shared, int threads, size_t smem) {
-  return occupancy_k(rollout_kernel_of(variant, general, shared, threads, false), threads, smem);
+int rollout_blocks_per_sm(int variant, bool general, int params, int threads, size_t smem) {
+  return occupancy_k(rollout_kernel_of(variant, general, params, threads, false), threads, smem);
 }
 
 // Two-environments-per-thread variants: 0: (288, 2)  1: (576, 1)  2: (1024, 1)  3: (288, 3)

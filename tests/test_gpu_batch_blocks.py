@@ -1,7 +1,7 @@
-"""The default block size of a heterogeneous batch where warp slots alone would
-ask for more groups a block than its shared memory holds: forward and reverse
-run, and each system's slice equals its solo launch (the tolerances of
-test_gpu_batch.py)."""
+"""The default block size of a heterogeneous batch of more blocks than are
+resident at once, where warp slots alone would ask for more groups a block than
+its shared memory holds: forward and reverse run, and each system's slice equals
+its solo launch (the tolerances of test_gpu_batch.py)."""
 import numpy as np
 import pytest
 
@@ -40,11 +40,11 @@ def chain(n, pairs=0):
 
 SETS = {
     # 32 warps by warp slots; the reverse of two 16-body groups takes 278,784 bytes
-    "20 + 16 bodies": lambda: [(chain(20), 64), (chain(16), 1024)],
+    "20 + 16 bodies": lambda: [(chain(20), 64), (chain(16), 8192)],
     # 27 warps by warp slots; the reverse of three quadruped groups takes 235,392 bytes
-    "20 bodies + quadruped": lambda: [(chain(20), 32), (S.quadruped(), 2048)],
+    "20 bodies + quadruped": lambda: [(chain(20), 32), (S.quadruped(), 16384)],
     # 18 warps by warp slots; the forward of two 9-body groups of 100 pairs takes 255,232 bytes
-    "17 + 9 bodies, pairs": lambda: [(chain(17, 20), 32), (chain(9, 100), 512)],
+    "17 + 9 bodies, pairs": lambda: [(chain(17, 20), 32), (chain(9, 100), 8192)],
 }
 
 

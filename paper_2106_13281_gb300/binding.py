@@ -18,6 +18,7 @@ LIB_PATH = os.path.join(HERE, "libbrax_gb300.so")
 BRAX_DESC_VERSION = 2
 STATUS = {0: "OK", 1: "INVALID_ARGUMENT", 2: "INVALID_DESCRIPTOR", 3: "CUDA", 4: "OUT_OF_MEMORY",
           5: "NONFINITE", 6: "TIMEOUT", 7: "WORKSPACE"}
+BRAX_ERR_WORKSPACE = 7
 
 # Every symbol include/brax.h declares.
 EXPORTS = ["brax_system_create", "brax_system_destroy", "brax_system_info", "brax_default_qp", "brax_step",

@@ -12,8 +12,8 @@ import os
 import numpy as np
 import torch
 
-from .binding import (BRAX_TUNE_FORWARD, BRAX_TUNE_REVERSE, _ptr, _stream, brax_tune_result, check, load_library,
-                      marshal_desc)
+from .binding import (BRAX_ERR_WORKSPACE, BRAX_TUNE_FORWARD, BRAX_TUNE_REVERSE, _ptr, _stream, brax_tune_result,
+                      check, load_library, marshal_desc)
 
 
 def _f32(t, shape=None, name="tensor"):
@@ -363,12 +363,22 @@ class BraxBatch:
         return w.value, ms.value
 
     def rollout_backward(self, state0, actions, checkpoints, g_state_T, T, K=1, g_torso=None, workspace=None):
+        """workspace: device scratch (uint8); one smaller than workspace_size
+        is used where brax_batch_rollout_backward takes it (at the price of
+        recomputed substeps), else replaced."""
         nbytes = self.workspace_size(T, K)
-        if workspace is None or workspace.numel() < nbytes:
+        if workspace is None:
             workspace = torch.empty((max(nbytes, 1),), device="cuda", dtype=torch.uint8)
         g_actions = torch.empty_like(actions)
         g_state0 = torch.empty_like(state0)
-        check(self._L.brax_batch_rollout_backward(self._h, T, K, _ptr(state0), _ptr(actions), _ptr(checkpoints),
-                                                  _ptr(g_state_T), _ptr(g_torso), _ptr(g_actions), _ptr(g_state0),
-                                                  _ptr(workspace), workspace.numel(), _stream()))
+
+        def run(ws):
+            return self._L.brax_batch_rollout_backward(self._h, T, K, _ptr(state0), _ptr(actions), _ptr(checkpoints),
+                                                       _ptr(g_state_T), _ptr(g_torso), _ptr(g_actions),
+                                                       _ptr(g_state0), _ptr(ws), ws.numel(), _stream())
+
+        code = run(workspace)
+        if code == BRAX_ERR_WORKSPACE and workspace.numel() < nbytes:
+            code = run(torch.empty((max(nbytes, 1),), device="cuda", dtype=torch.uint8))
+        check(code)
         return g_actions, g_state0

@@ -90,3 +90,20 @@ def test_batch_gradients_do_not_depend_on_the_workspace(systems, names, T, K):
         outs.append((ga, gs))
         assert b._L.brax_batch_rollout_backward(*args, 4096, _stream()) == 7
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+def test_a_smaller_batch_workspace_is_used(systems):
+    """BraxBatch.rollout_backward runs in a smaller workspace than it asks for
+    instead of allocating the full one, and replaces one too small to run in."""
+    T, K = 4, 4
+    b, st, a, ck = batch_of(systems, T, K)
+    g, need = torch.ones_like(st), b.workspace_size(T, K)
+    ref = b.rollout_backward(st, a, ck, g, T, K=K)
+    for nbytes, allocates in ((need - 256, False), (256, True)):
+        ws = torch.empty(nbytes, device="cuda", dtype=torch.uint8)
+        torch.cuda.synchronize()
+        torch.cuda.reset_peak_memory_stats()
+        before = torch.cuda.memory_allocated()
+        got = b.rollout_backward(st, a, ck, g, T, K=K, workspace=ws)
+        assert (torch.cuda.max_memory_allocated() - before >= need) == allocates
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])

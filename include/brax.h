@@ -175,7 +175,10 @@ int brax_step(const brax_system* sys, int64_t n_envs, const float* state_in, con
  * autotuner found the one-environment kernel faster; checkpointing rollouts
  * run the same kernel, and brax_rollout_backward rebuilds step states with
  * the kernel that wrote the checkpoints, so gradients do not depend on K.
- * The two kernels agree to FP32 rounding.
+ * The two kernels agree to FP32 rounding.  Of these systems, those of one root
+ * (body 0) with 1, 2, 4 or 8 limbs of two bodies each, alike but for their
+ * geometry, on z-up ground, run a limb or a limb body per thread where that is
+ * faster; these kernels give the bits of the two-environments kernel.
  * Schedule: a block keeps its environments on chip for the whole rollout,
  * so when the blocks are not a whole number of resident waves the last wave
  * would run part-empty from the first step to the last.  Then the rollout of

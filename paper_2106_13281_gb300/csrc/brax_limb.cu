@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(128, 2) rollout_limb_kernel(const __grid_const
         integrate(S2, average, fr_, qr, wr, sr, fr, acc);
       }
     }
-    if (sg.torso && br == 0 && limb == 0) {
+    if (sg.torso && br == 0 && limb == 0) {  // (the root is body 0; without the test the code came out slower)
       float* tp = sg.torso + (int64_t)t * N * 3;
       if (va) {
         tp[ea * 3 + 0] = sr.x.x.x;
@@ -449,10 +449,10 @@ __device__ __forceinline__ void contacts_first(const SysP2& S2, bool average, Fl
 // Few environments leave a warp alone on its SM sub-partition, where a substep
 // lasts as long as one warp takes: the wide kernel's lane does a whole limb of
 // two environments (1,260 instructions a substep), this one's a body of one
-// (560), with the contact responses in straight code beside the joint's.
-// Quadruped, us a step: up to 2,048 environments 5.4 (paired 18), 4,096 9.2
-// (18), 8,192 14.8 (18), 12,288 22.2 (27), 16,384 29.2 (28).  Its root is computed by 2 L lanes, the wide
-// kernel's by L / 2 per environment, so it loses where warps fill the SMs.
+// (560), with the contact responses in straight code beside the joint's.  Its
+// root is computed by 2 L lanes, the wide kernel's by L / 2 per environment, so
+// it loses where warps fill the SMs (us a step of both and of the body layout:
+// the table at limb_rule in brax_capi.cu).
 //
 // kFew: at most 8 warps an SM, no spills (36 bytes under the 168 registers that
 // let 12 be resident, which more warps need).  With the start's loads taken

@@ -20,8 +20,6 @@
 
 namespace brax {
 
-constexpr int kMaxLimbs = BRAX_MAX_CHILDREN;
-
 // A limb body's geometry in shared memory, as (value, value) pairs: the
 // parameters that differ from limb to limb.  The scalars, alike for all limbs,
 // are read from the constant pool.

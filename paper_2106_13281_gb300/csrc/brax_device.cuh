@@ -241,15 +241,18 @@ __device__ __forceinline__ void bar_arrive(int id, int nthreads) {
 // constant pool, the pairs' from shared memory, or the bodies', pairs' and
 // planes'.
 enum ParamsIn : int { kInPool = 0, kPairsShared = 1, kAllShared = 2 };
-// Copy a system's pair parameters, or its body, pair and plane parameters (what
-// follows SysP in its blob), to shared memory; the whole block takes part, and
+// Copy a system's body, pair and plane parameters (what follows SysP in its
+// blob), or the pairs' alone, to shared memory; the whole block takes part, and
 // synchronises after.
-template <int kParams>
 __device__ __forceinline__ void copy_params(const unsigned char* blob, unsigned char* dst, int B, int P, int n_planes) {
-  const uint4* src = reinterpret_cast<const uint4*>(blob + (kParams == kAllShared ? blob_bodies_off() : blob_pairs_off(B)));
-  const int bytes = kParams == kAllShared ? params_bytes(B, P, n_planes) : P * (int)sizeof(PairP);
+  const uint4* src = reinterpret_cast<const uint4*>(blob + blob_bodies_off());
   uint4* d = reinterpret_cast<uint4*>(dst);
-  for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) d[i] = __ldg(src + i);
+  for (int i = threadIdx.x; i < params_bytes(B, P, n_planes) / 16; i += blockDim.x) d[i] = __ldg(src + i);
+}
+__device__ __forceinline__ void copy_pairs(const unsigned char* blob, unsigned char* dst, int B, int P) {
+  const uint4* src = reinterpret_cast<const uint4*>(blob + blob_pairs_off(B));
+  uint4* d = reinterpret_cast<uint4*>(dst);
+  for (int i = threadIdx.x; i < P * (int)(sizeof(PairP) / 16); i += blockDim.x) d[i] = __ldg(src + i);
 }
 static_assert(sizeof(PairP) % 16 == 0 && sizeof(BodyP) % 16 == 0, "the pairs are copied as 16-byte words");
 

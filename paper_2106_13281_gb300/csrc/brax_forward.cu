@@ -124,14 +124,18 @@ __global__ void __launch_bounds__(MAXT, MINB) rollout_kernel(const __grid_consta
   const Seg& sg = L.seg[si];
   const unsigned char* blob = c_pool + sg.pool_off;
   const SysP& S = *reinterpret_cast<const SysP*>(blob);
-  unsigned char* const params = smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float);
-  if constexpr (kParams != kInPool) {
-    copy_params<kParams>(sg.blob, params, sg.B, sg.P, S.n_planes);
+  if constexpr (kParams == kAllShared) {
+    blob = smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float) - sizeof(SysP);
+    copy_params(sg.blob, smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P, S.n_planes);
+    group_sync(0, blockDim.x);
+  } else if constexpr (kParams == kPairsShared) {
+    copy_pairs(sg.blob, smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float), sg.B, sg.P);
     group_sync(0, blockDim.x);
   }
-  if constexpr (kParams == kAllShared) blob = params - sizeof(SysP);
   const BodyP* bodies = reinterpret_cast<const BodyP*>(blob + blob_bodies_off());
-  const PairP* pairs = reinterpret_cast<const PairP*>(kParams == kPairsShared ? params : blob + blob_pairs_off(sg.B));
+  const PairP* pairs = reinterpret_cast<const PairP*>(blob + blob_pairs_off(sg.B));
+  if constexpr (kParams == kPairsShared)
+    pairs = reinterpret_cast<const PairP*>(smem + sg.groups * group_floats(sg.B, sg.P) * sizeof(float));
   const PlaneP* planes = reinterpret_cast<const PlaneP*>(blob + blob_planes_off(sg.B, sg.P));
   const int B = sg.B;
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);

@@ -805,7 +805,7 @@ struct SchedHold {
   cudaEvent_t done = nullptr;
   cudaStream_t st = nullptr;
   ~SchedHold() {
-    if (done) cudaEventRecord(done, st);
+    if (done && cudaEventRecord(done, st) != cudaSuccess) cudaGetLastError();
   }
 };
 bool is_capturing(cudaStream_t st) {

@@ -12,8 +12,8 @@ import os
 import numpy as np
 import torch
 
-from .binding import (BRAX_ERR_WORKSPACE, BRAX_TUNE_FORWARD, BRAX_TUNE_REVERSE, _ptr, _stream, brax_tune_result,
-                      check, load_library, marshal_desc)
+from .binding import (BRAX_ERR_WORKSPACE, BRAX_TUNE_FORWARD, BRAX_TUNE_REVERSE, BraxError, _ptr, _stream,
+                      brax_tune_result, check, load_library, marshal_desc)
 
 
 def _f32(t, shape=None, name="tensor"):
@@ -113,17 +113,8 @@ class BraxSystem:
         if cache and os.path.exists(cache):
             with open(cache) as fh:
                 table = json.load(fh)
-        if key in table:
-            r = table[key]
-            if forward:
-                self.set_launch(r["scalar_groups"], r["scalar_variant"])
-                if r["fwd_kernel"] == 1:
-                    self.set_pair_launch(1, r["fwd_groups"], r["fwd_variant"])
-                elif self.paired:
-                    self.set_pair_launch(0)
-            if r.get("bwd_variant", -1) >= 0:
-                self._L.brax_system_set_backward_launch(self._h, r["bwd_variant"])
-            return dict(r, cached=True)
+        if key in table and self._apply_tuning(table[key], forward):
+            return dict(table[key], cached=True)
         out = brax_tune_result()
         check(self._L.brax_autotune(self._h, N, T, _ptr(state0), _ptr(actions), flags, mem_budget, _stream(),
                                     C.byref(out)))
@@ -138,6 +129,23 @@ class BraxSystem:
                 json.dump(table, fh, indent=1)
             os.replace(tmp, cache)
         return dict(r, cached=False)
+
+    def _apply_tuning(self, r: dict, forward: bool) -> bool:
+        """Apply a cached configuration; False where it names a launch that
+        this system does not have (the limb layout of a system it no longer
+        takes): it is then tuned anew."""
+        try:
+            if forward:
+                self.set_launch(r["scalar_groups"], r["scalar_variant"])
+                if r["fwd_kernel"] == 1:
+                    self.set_pair_launch(1, r["fwd_groups"], r["fwd_variant"])
+                elif self.paired:
+                    self.set_pair_launch(0)
+        except BraxError:
+            return False
+        if r.get("bwd_variant", -1) >= 0:
+            self._L.brax_system_set_backward_launch(self._h, r["bwd_variant"])
+        return True
 
     def last_rollout(self) -> dict:
         """Launch of the last rollout: blocks, chunks of the chunked schedule

@@ -103,3 +103,20 @@ def test_environment_layer_of_a_jointed_body_0(brax, name, drop, mode):
         assert np.abs(rew - exp).max() < 1e-5 * (1.0 + np.abs(exp).max())
         st = out["state_T"]
     sysm.sync_status()
+
+
+def test_a_cached_limb_launch_is_tuned_anew(brax, tmp_path):
+    """An autotune cache that recorded the limb layout for a system whose root
+    is not body 0 is not applied: the system is tuned again."""
+    import json
+    r, order = root_last(S.quadruped())
+    sysm, cache = brax(r), str(tmp_path / "tune.json")
+    st, a = inputs(brax, S.quadruped(), order, 64, 4, 0.36)
+    first = sysm.autotune(st, a, cache=cache)
+    table = json.load(open(cache))
+    (key,) = table
+    table[key].update(fwd_kernel=1, fwd_groups=1, fwd_variant=5)
+    json.dump(table, open(cache, "w"))
+    again = sysm.autotune(st, a, cache=cache)
+    assert not first["cached"] and not again["cached"] and again["fwd_variant"] < 5
+    assert sysm.autotune(st, a, cache=cache)["cached"]

@@ -588,7 +588,7 @@ bool fits_block(size_t with, int device) {
 // pairs' and with all parameters behind the groups.
 //
 // Shared memory serves what the constant cache misses: the biped's substep takes
-// 6.7 us with all parameters there and 10.8 from the pool (4,864 environments,
+// 6.0 us with all parameters there and 9.5 from the pool (4,864 environments,
 // one group an SM).  But an SM's shared memory is cut from its L1 cache in steps
 // (carve-outs), and the kernels spill registers (190 to 340 bytes a thread) to
 // L1: a launch whose bodies' parameters take the SM a step further pays more for

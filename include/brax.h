@@ -25,8 +25,8 @@
  *  - Device memory for a system's parameters and its status word is
  *    allocated once by brax_system_create; the reverse pass's workspace comes
  *    from the caller (brax_workspace_size).  The one allocation a compute
- *    call can make is the chunked schedule's scratch (a ring of four regions
- *    of (32 + blocks) int32, a few KB): brax_rollout, brax_rollout_backward
+ *    call can make is the chunked schedule's scratch (eight regions of
+ *    (32 + blocks) int32, a few KB, and four events): brax_rollout, brax_rollout_backward
  *    and the batch rollouts allocate it the first time a launch takes the
  *    chunked schedule (see brax_rollout) or needs a larger one; a call made
  *    while its stream is being captured takes the static schedule instead of
